@@ -42,6 +42,7 @@
 #define __forceinline__ inline
 #endif
 
+#include "arith64.cuh"
 #include "convert.cuh"
 
 namespace osiris_explog {
@@ -103,12 +104,13 @@ constexpr long long kShiftBits = 0x4338000000000000LL;
 // 1/3 as a float pair, for the log1p series
 constexpr float kThirdH = 0.3333333432674408f, kThirdL = -9.934107758624577e-09f;
 
-__device__ __forceinline__ double exp_tab(double y, const double* t2) {
+template <class A = osiris_impl::ArithPlain>
+__device__ __forceinline__ double exp_tab(double y, const double* t2, A&& ar = A()) {
   using namespace osiris_impl;
   if (!(fabs(y) < 700.0)) return exp(y);
   const double t = fma(y, kInvL, kShift);
   const int n = (int)(to_bits(t) & 0xffffffffLL);  // y * 64/ln2 rounded, mod 2^32
-  const double nd = t - kShift;
+  const double nd = ar.sub(t, kShift);
   const double r = fma(-nd, kL2, fma(-nd, kL1, y));
   // exp(r) - 1 = r + c, c = r^2 (1/2 + r/6 + r^2/24 + r^3/120), in double-float:
   // the r/6 term as a product with 1/6 in two words, the rest in FP32
@@ -117,13 +119,14 @@ __device__ __forceinline__ double exp_tab(double y, const double* t2) {
   const float small = __fmul_rn(__fmul_rn(rf, rf), fmaf(rf, 1.0f / 120.0f, 1.0f / 24.0f));
   const df q = df_add_f_u(df_add_f_u(df_mul(rd, mk(dfc::I3H, dfc::I3L)), small), 0.5f);
   const df c = df_mul(df_sqr(rd), q);
-  const double p = (r + float_to_double0(c.hi)) + float_to_double0(c.lo);
+  const double p = ar.add(ar.add(r, float_to_double0(c.hi)), float_to_double0(c.lo));
   const double T = t2[n & (kExpN - 1)];
   const double e = fma(T, p, T);  // in [0.99, 2.02): scaling by 2^m stays normal
   return from_bits(to_bits(e) + (long long)(n >> 6) * (1LL << 52));
 }
 
-__device__ __forceinline__ double log_tab(double x, const LogEntry* lg) {
+template <class A = osiris_impl::ArithPlain>
+__device__ __forceinline__ double log_tab(double x, const LogEntry* lg, A&& ar = A()) {
   using namespace osiris_impl;
   if (!(x >= 0x1p-1000 && x <= 0x1p+1000)) return log(x);
   const long long b = to_bits(x);
@@ -132,7 +135,7 @@ __device__ __forceinline__ double log_tab(double x, const LogEntry* lg) {
   const int j = ((hi & 0xfffff) + 0x1000) >> 13;  // nearest multiple of 1/128, 0..128
   const double F = from_bits(0x3ff0000000000000LL + ((long long)j << 45));
   const LogEntry E = lg[j];
-  const double u = (m - F) * E.rcpF;  // m - F is exact
+  const double u = ar.mul(ar.sub(m, F), E.rcpF);  // m - F is exact
   // log1p(u) = u + c, c = u^2 (-1/2 + u/3 - u^2/4 + u^3/5 - u^4/6 + u^5/7), in
   // double-float. The result is ~u, so c needs ~2^-53 / |u| relative accuracy:
   // the u/3 and u^2/4 terms in two words, from u^3 on in FP32.
@@ -145,10 +148,10 @@ __device__ __forceinline__ double log_tab(double x, const LogEntry* lg) {
       df_add_f_u(df_add_u(df_mul(ud, mk(kThirdH, kThirdL)), df_scale(usq, -0.25f)), small),
       -0.5f);
   const df c = df_mul(usq, q);
-  const double l1p = (u + float_to_double0(c.hi)) + float_to_double0(c.lo);
+  const double l1p = ar.add(ar.add(u, float_to_double0(c.hi)), float_to_double0(c.lo));
   const int k = (hi >> 20) - 1023 + (j >= kLogHalf ? 1 : 0);
-  const double kd = from_bits(kShiftBits + k) - kShift;
-  return fma(kd, kLn2Hi, E.logF) + fma(kd, kLn2Lo, l1p);
+  const double kd = ar.sub(from_bits(kShiftBits + k), kShift);
+  return ar.add(fma(kd, kLn2Hi, E.logF), fma(kd, kLn2Lo, l1p));
 }
 
 }  // namespace osiris_explog

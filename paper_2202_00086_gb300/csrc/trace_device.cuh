@@ -21,6 +21,7 @@
 
 #include <cstdint>
 
+#include "arith64.cuh"
 #include "convert.cuh"
 #include "df64.cuh"
 #include "explog.cuh"
@@ -146,6 +147,26 @@ __device__ __forceinline__ void trig_table_init() {
   __syncthreads();
 }
 
+// The block's 1 and -0, the vector operands of ArithFast (arith64.cuh): read
+// from shared memory, no compiler pass knows their values.
+struct FmaUnits {
+  double one, nz;
+};
+
+__device__ __forceinline__ volatile FmaUnits& fma_units() {
+  __shared__ FmaUnits u;
+  return u;
+}
+
+// All threads of the block, before any divergence.
+__device__ __forceinline__ void fma_units_init() {
+  if (threadIdx.x == 0) {
+    fma_units().one = 1.0;
+    fma_units().nz = -0.0;
+  }
+  __syncthreads();
+}
+
 // The block's copy of the exp/log breakpoint tables (explog.cuh), filled by
 // all threads of the block before any divergence.
 __device__ __forceinline__ osiris_explog::Tables& explog_table() {
@@ -200,7 +221,8 @@ __device__ __forceinline__ float add_as_fma(float a, float c) { return a + c; }
 
 
 
-__device__ __forceinline__ void sincos_tab(double th, double& s, double& c) {
+template <class A = ArithPlain>
+__device__ __forceinline__ void sincos_tab(double th, double& s, double& c, A&& ar = A()) {
   using namespace dfc;
   // nearest node in FP32: 1.5 * 2^23 added to round to an integer
   const float tk = fmaf(to_float_rz(th), (float)(kTrigPerPi / 3.14159265358979323846),
@@ -213,7 +235,7 @@ __device__ __forceinline__ void sincos_tab(double th, double& s, double& c) {
   const TrigTable& t = trig_table();
   const double2 sc = t.sc[idx];
   const float4 scf = t.scf[idx];
-  const double x = th - t.n[idx];  // exact
+  const double x = ar.sub(th, t.n[idx]);  // exact
   // the corrections in double-float
   const df xd = split_df(x);
   const df u = df_sqr(xd);                                                    // x^2
@@ -224,8 +246,10 @@ __device__ __forceinline__ void sincos_tab(double th, double& s, double& c) {
   const df S = mk(scf.x, scf.y), C = mk(scf.z, scf.w);
   const df corr_s = df_add_u(df_mul(C, ds), df_mul(S, cm));
   const df corr_c = df_sub_u(df_mul(C, cm), df_mul(S, ds));
-  s = fma(sc.y, x, sc.x + float_to_double0(corr_s.hi)) + float_to_double0(corr_s.lo);
-  c = fma(-sc.x, x, sc.y + float_to_double0(corr_c.hi)) + float_to_double0(corr_c.lo);
+  s = ar.add(fma(sc.y, x, ar.add(sc.x, float_to_double0(corr_s.hi))),
+             float_to_double0(corr_s.lo));
+  c = ar.add(fma(-sc.x, x, ar.add(sc.y, float_to_double0(corr_c.hi))),
+             float_to_double0(corr_c.lo));
 }
 
 // max |H - H0| kept as the bit pattern of a non-negative double: |v| and the
@@ -238,7 +262,8 @@ __device__ __forceinline__ void track_abs_H(long long& max_bits, double twoH, do
 // 1/d: FP32 seed x0 (|x0 d - 1| < 2^-21), then one Newton step with the
 // cubic term, x0 (1 + e + e^2) with e = 1 - d x0, relative error e^3 plus
 // the final rounding (3 FP64 instructions). Outside the FP32 range: 1/d.
-__device__ __forceinline__ double rcp64(double d) {
+template <class A = ArithPlain>
+__device__ __forceinline__ double rcp64(double d, A&& ar = A()) {
   const long long b = __double_as_longlong(d);
   const int e = (int)((b >> 52) & 0x7ff) - 1023 + 127;
   if (e < 2 || e > 252) return 1.0 / d;
@@ -251,7 +276,7 @@ __device__ __forceinline__ double rcp64(double d) {
   rf = 1.0f / f;  // host builds of this header (CPU tests): a correctly rounded seed
 #endif
   const double x0 = float_to_double(rf);
-  const double eps = fma(-d, x0, 1.0);
+  const double eps = fma(-d, x0, ar.unit());
   return fma(x0, fma(eps, eps, eps), x0);
 }
 
@@ -279,39 +304,49 @@ __device__ __forceinline__ double rcp64(double d) {
 // Y = p_r^2 + u^2, L / sin reused). twoH receives 2H = N / Sigma at the
 // evaluation point.
 // ---------------------------------------------------------------------------
+// With ArithFast the products of factors that ordinary rays keep away from
+// zero go to the integer pipes; the others may vanish (a = 0, L = 0, cos = 0)
+// and stay on the FP64 unit.
+template <class A = ArithPlain>
 __device__ __forceinline__ void rhs64(const RayK& K, double r, double th, double pr, double pth,
                                       double& dr, double& dth, double& dph, double& dpr,
-                                      double& dpth, double& twoH, double& scale) {
+                                      double& dpth, double& twoH, double& scale, A&& ar = A()) {
   double s, c;
-  sincos_tab(th, s, c);
+  sincos_tab(th, s, c, ar);
   const double ra2 = fma(r, r, K.a2);  // r^2 + a^2
-  const double a2s = K.a2 * s;
-  const double Delta = fma(r, r - 2.0, K.a2);
+  const double a2s = ar.mul(K.a2, s);
+  const double Delta = fma(r, ar.sub(r, 2.0), K.a2);
   // Sigma = r^2 + a^2 cos^2 = (r^2 + a^2) - a^2 sin^2 (no cancellation: r > a)
   const double Sigma = fma(-a2s, s, ra2);
   const double P = fma(ra2, K.E, -K.aL);
-  const double DS = Delta * Sigma;
-  const double inv = rcp64(DS * s);
-  const double sinv = s * inv;  // 1 / (Delta Sigma)
-  const double iSig = Delta * sinv;
-  const double iDel = Sigma * sinv;
-  const double is = DS * inv;
-  const double Lis = K.L * is;  // L / sin
+  ar.window(s);
+  ar.window(Delta);
+  ar.window(Sigma);
+  ar.window(P);
+  ar.window(pr);
+  const double DS = ar.soft(Delta, Sigma);
+  const double inv = rcp64(ar.soft(DS, s), ar);
+  const double sinv = ar.soft(s, inv);  // 1 / (Delta Sigma)
+  const double iSig = ar.soft(Delta, sinv);
+  const double iDel = ar.soft(Sigma, sinv);
+  const double is = ar.soft(DS, inv);
+  const double Lis = ar.mul(K.L, is);  // L / sin
   const double W = fma(-K.aE, s, Lis);
-  const double u = P * iDel;
-  const double Dpr = Delta * pr;
-  const double N = fma(Dpr, pr, fma(pth, pth, fma(W, W, -P * u)));
-  const double NiS = N * iSig;
+  const double u = ar.soft(P, iDel);
+  const double Dpr = ar.soft(Delta, pr);
+  const double N = fma(Dpr, pr, fma(pth, pth, fma(W, W, -ar.soft(P, u))));
+  ar.window(N);
+  const double NiS = ar.soft(N, iSig);
   // Every derivative carries the factor 1/Sigma; it is returned separately
   // (scale) and folded into the stepper's tableau coefficients.
   dr = Dpr;
   dth = pth;
-  dph = fma(W, is, K.a * u);
+  dph = fma(W, is, ar.mul(K.a, u));
   // -dH/dr: (1 - r) Y + r X = Y + r (X - Y), Y = u^2 + p_r^2, X = 2H + 2E u
-  const double Y = fma(u, u, pr * pr);
-  dpr = fma(r, fma(K.E2, u, NiS) - Y, Y);
+  const double Y = fma(u, u, ar.soft(pr, pr));
+  dpr = fma(r, ar.sub(fma(K.E2, u, NiS), Y), Y);
   // -dH/dtheta: cos (W (L / sin^2 + a E) - a^2 sin 2H)
-  dpth = c * fma(W, fma(Lis, is, K.aE), -a2s * NiS);
+  dpth = ar.mul(c, fma(W, fma(Lis, is, K.aE), -ar.mul(a2s, NiS)));
   scale = iSig;
   twoH = NiS;
 }
@@ -328,49 +363,64 @@ __device__ __forceinline__ void rhs64(const RayK& K, double r, double th, double
 // The powers f^q and X^k come from the table-driven exp and log of
 // explog.cuh (about a third of the library's FP64 instructions).
 // ---------------------------------------------------------------------------
+template <class A = ArithPlain>
 __device__ __forceinline__ void rhs_q64(const RayK& K, double r, double th, double pr,
                                         double pth, double& dr, double& dth, double& dph,
-                                        double& dpr, double& dpth, double& twoH, double& scale) {
+                                        double& dpr, double& dpth, double& twoH, double& scale,
+                                        A&& ar = A()) {
   scale = 1.0;
   double s, c;
-  sincos_tab(th, s, c);
+  sincos_tab(th, s, c, ar);
   // four reciprocals (1/D, 1/X, 1/sin^2, 1/(f f^q)) serve every quotient:
   // 1/r = (r - 2)/D, and f = (r - 2)/r keeps its relative accuracy at r -> 2
-  const double rm2 = r - 2.0;
-  const double iD = rcp64(r * rm2);
-  const double ir = rm2 * iD;
-  const double f = rm2 * ir;
-  const double s2 = s * s;
-  const double is2 = rcp64(s2);
-  const double X = fma(s2, iD, 1.0);
-  const double iX = rcp64(X);
+  const double rm2 = ar.sub(r, 2.0);
+  ar.window(r);
+  ar.window(rm2);
+  ar.window(s);
+  ar.window(c);
+  ar.window(pr);
+  const double iD = rcp64(ar.soft(r, rm2), ar);
+  const double ir = ar.soft(rm2, iD);
+  const double f = ar.soft(rm2, ir);
+  const double s2 = ar.soft(s, s);
+  const double is2 = rcp64(s2, ar);
+  const double X = fma(s2, iD, ar.unit());
+  const double iX = rcp64(X, ar);
   const osiris_explog::Tables& T = explog_table();
-  const double fq = osiris_explog::exp_tab(K.q * osiris_explog::log_tab(f, T.lg), T.t2);
-  const double Xk = osiris_explog::exp_tab(K.kap * osiris_explog::log_tab(X, T.lg), T.t2);
-  const double ir2 = ir * ir;
-  const double ffq = f * fq;
-  const double fXk = fq * Xk;
-  const double gtt = -rcp64(ffq);
-  const double grr = f * fXk;
-  const double gthth = fXk * ir2;
-  const double gpp = fq * ir2 * is2;
-  dr = grr * pr;
-  dth = gthth * pth;
-  dph = gpp * K.L;
+  const double fq =
+      osiris_explog::exp_tab(ar.mul(K.q, osiris_explog::log_tab(f, T.lg, ar)), T.t2, ar);
+  const double Xk =
+      osiris_explog::exp_tab(ar.mul(K.kap, osiris_explog::log_tab(X, T.lg, ar)), T.t2, ar);
+  ar.window(fq);
+  ar.window(Xk);
+  ar.window(X);
+  const double ir2 = ar.soft(ir, ir);
+  const double ffq = ar.soft(f, fq);
+  const double fXk = ar.soft(fq, Xk);
+  const double gtt = -rcp64(ffq, ar);
+  const double grr = ar.soft(f, fXk);
+  const double gthth = ar.soft(fXk, ir2);
+  const double gpp = ar.soft(ar.soft(fq, ir2), is2);
+  dr = ar.soft(grr, pr);
+  dth = ar.mul(gthth, pth);
+  dph = ar.mul(gpp, K.L);
   // the four terms of 2H
-  const double Ht = gtt * (K.E * K.E), Hr = dr * pr, Hth = dth * pth, Hph = dph * K.L;
-  twoH = (Ht + Hr) + (Hth + Hph);
+  const double Ht = ar.mul(gtt, ar.mul(K.E, K.E)), Hr = ar.soft(dr, pr), Hth = ar.mul(dth, pth),
+               Hph = ar.mul(dph, K.L);
+  twoH = ar.add(ar.add(Ht, Hr), ar.add(Hth, Hph));
   // -dH/dr = -1/2 sum_mu (d ln g^mumu / dr) H_mu, collected by logarithmic
   // derivative: -1/2 [(1+q) d ln f (Hr - Ht) + k d ln X (Hr + Hth)
   //                   + (q d ln f - 2/r) (Hth + Hph)]
-  const double iDX = iD * iX;
-  const double a1 = fma(-K.q, iD, -iD);                 // -(1+q)/D
-  const double a2 = K.kap * s2 * (r - 1.0) * iD * iDX;  // k sin^2 (r-1) / (D^2 X)
-  const double a3 = fma(-K.q, iD, ir);                  // 1/r - q/D
-  dpr = fma(a1, Hr - Ht, fma(a2, Hr + Hth, a3 * (Hth + Hph)));
+  const double iDX = ar.soft(iD, iX);
+  const double HrHth = ar.add(Hr, Hth);
+  const double a1 = fma(-K.q, iD, -iD);  // -(1+q)/D
+  // k sin^2 (r-1) / (D^2 X)
+  const double a2 = ar.mul(ar.mul(ar.mul(ar.mul(K.kap, s2), ar.sub(r, 1.0)), iD), iDX);
+  const double a3 = fma(-K.q, iD, ir);  // 1/r - q/D
+  dpr = fma(a1, ar.sub(Hr, Ht), fma(a2, HrHth, ar.mul(a3, ar.add(Hth, Hph))));
   // -dH/dtheta = -1/2 (k d ln X/dtheta (Hr + Hth) - 2 (cos/sin) Hph)
   //            = sin cos (Hph / sin^2 - k (Hr + Hth) / (D X))
-  dpth = (c * s) * fma(-K.kap * iDX, Hr + Hth, Hph * is2);
+  dpth = ar.mul(ar.soft(c, s), fma(ar.mul(-K.kap, iDX), HrHth, ar.mul(Hph, is2)));
 }
 
 // Metric policies for the FP64 steppers.
@@ -386,22 +436,26 @@ struct KerrMetric {
   // 2.95 at 168 registers (three blocks) and 2.90 at 152 or 128 (three or
   // four blocks). The FP64 pipe needs the scheduling freedom more than warps.
   static constexpr int kMaxRegs = OSIRIS_FP64_MAXREGS;
+  static constexpr bool kUnitScale = false;
+  template <class A>
   static __device__ __forceinline__ void rhs(const RayK& K, double r, double th, double pr,
                                              double pth, double& dr, double& dth, double& dph,
                                              double& dpr, double& dpth, double& twoH,
-                                             double& scale) {
-    rhs64(K, r, th, pr, pth, dr, dth, dph, dpr, dpth, twoH, scale);
+                                             double& scale, A& ar) {
+    rhs64(K, r, th, pr, pth, dr, dth, dph, dpr, dpth, twoH, scale, ar);
   }
 };
 struct QMetric {
   static constexpr bool kTrigTable = true;  // rhs_q64 reads the block's sincos table
   static constexpr bool kExpLogTable = true;  // and the exp/log tables
   static constexpr int kMaxRegs = OSIRIS_FP64_MAXREGS;
+  static constexpr bool kUnitScale = true;
+  template <class A>
   static __device__ __forceinline__ void rhs(const RayK& K, double r, double th, double pr,
                                              double pth, double& dr, double& dth, double& dph,
                                              double& dpr, double& dpth, double& twoH,
-                                             double& scale) {
-    rhs_q64(K, r, th, pr, pth, dr, dth, dph, dpr, dpth, twoH, scale);
+                                             double& scale, A& ar) {
+    rhs_q64(K, r, th, pr, pth, dr, dth, dph, dpr, dpth, twoH, scale, ar);
   }
 };
 
@@ -413,15 +467,15 @@ struct Deriv {
   double scale, twoH;
 };
 
-template <class Met = KerrMetric>
+template <class Met = KerrMetric, class A = ArithPlain>
 __device__ __forceinline__ void rhs64_at(const RayK& K, double r, double th, double pr,
-                                         double pth, Deriv& k) {
-  Met::rhs(K, r, th, pr, pth, k.r, k.th, k.ph, k.pr, k.pth, k.twoH, k.scale);
+                                         double pth, Deriv& k, A&& ar = A()) {
+  Met::rhs(K, r, th, pr, pth, k.r, k.th, k.ph, k.pr, k.pth, k.twoH, k.scale, ar);
 }
 
-template <class Met = KerrMetric>
-__device__ __forceinline__ void rhs64_at(const RayK& K, const State& y, Deriv& k) {
-  rhs64_at<Met>(K, y.r, y.th, y.pr, y.pth, k);
+template <class Met = KerrMetric, class A = ArithPlain>
+__device__ __forceinline__ void rhs64_at(const RayK& K, const State& y, Deriv& k, A&& ar = A()) {
+  rhs64_at<Met>(K, y.r, y.th, y.pr, y.pth, k, ar);
 }
 
 // 2H at a state (used once per ray for the terminal point).
@@ -432,73 +486,139 @@ __device__ __forceinline__ double twoH64(const RayK& K, const State& y) {
   return k.twoH;
 }
 
-// Embedded Runge-Kutta attempt of length h from y with the tableau T (FP64
-// everywhere): o = fifth-order result, d = fifth minus fourth order. The
-// stage derivative k_j = scale_j * k~_j enters every sum through the
-// coefficient T.a[s][j] * (h scale_j), so the evaluations never multiply their
-// outputs by 1/Sigma; the stage inputs and o are accumulated directly onto y
-// (a few ulp of |y| per step, far below the truncation error at any usable
-// tolerance). phi is cyclic: its stage values are never needed, only its
-// increment. With FSAL the last stage is evaluated at o itself and k[NS - 1]
-// is the first stage of the next step.
-template <int NS>
-struct Tableau64 {
-  double a[NS][NS];  // a[s][j], j < s
-  double b[NS];      // fifth-order weights
-  double e[NS];      // fifth minus embedded fourth order
+// Embedded Runge-Kutta attempt of length h from y (FP64 everywhere): o =
+// fifth-order result, d = fifth minus fourth order. The stage derivative
+// k_j = scale_j * k~_j enters every sum through the coefficient
+// T.a[s][j] * (h scale_j), so the evaluations never multiply their outputs by
+// 1/Sigma; the stage inputs and o are accumulated directly onto y (a few ulp
+// of |y| per step, far below the truncation error at any usable tolerance).
+// phi is cyclic: its stage values are never needed, only its increment. With
+// FSAL the last stage is evaluated at o itself and is the first stage of the
+// next step.
+
+// The rows a[s][j], j < s, where the rolled stage loop can index them.
+#ifdef __CUDACC__
+#define OSIRIS_TABLEAU64 static __constant__
+#else
+#define OSIRIS_TABLEAU64 static const
+#endif
+OSIRIS_TABLEAU64 double kCashKarpA[6][6] = {
+    {0, 0, 0, 0, 0, 0},
+    {ck::A21, 0, 0, 0, 0, 0},
+    {ck::A31, ck::A32, 0, 0, 0, 0},
+    {ck::A41, ck::A42, ck::A43, 0, 0, 0},
+    {ck::A51, ck::A52, ck::A53, ck::A54, 0, 0},
+    {ck::A61, ck::A62, ck::A63, ck::A64, ck::A65, 0}};
+OSIRIS_TABLEAU64 double kDormandPrinceA[6][6] = {
+    {0, 0, 0, 0, 0, 0},
+    {dp::A21, 0, 0, 0, 0, 0},
+    {dp::A31, dp::A32, 0, 0, 0, 0},
+    {dp::A41, dp::A42, dp::A43, 0, 0, 0},
+    {dp::A51, dp::A52, dp::A53, dp::A54, 0, 0},
+    {dp::A61, dp::A62, dp::A63, dp::A64, dp::A65, 0}};  // the seventh stage is evaluated at o
+#undef OSIRIS_TABLEAU64
+
+struct CashKarp64 {
+  static constexpr int kStages = 6;
+  static constexpr bool kFsal = false;
+  static __device__ __forceinline__ double a(int s, int j) { return kCashKarpA[s][j]; }
+  static __device__ constexpr double b(int j) {  // fifth-order weights
+    constexpr double B[6] = {ck::B1, 0, ck::B3, ck::B4, 0, ck::B6};
+    return B[j];
+  }
+  static __device__ constexpr double e(int j) {  // fifth minus embedded fourth order
+    constexpr double E[6] = {ck::D1, 0, ck::D3, ck::D4, ck::D5, ck::D6};
+    return E[j];
+  }
 };
 
-// Stages 1 .. NS-1 (stage 0, k[0], is given), o and d. FSAL: the last
-// stage is evaluated at o.
-template <class Met, int NS, bool FSAL>
-__device__ __forceinline__ void rk_attempt64(const Tableau64<NS>& T, const RayK& K,
-                                             const State& y, double h, Deriv (&k)[NS],
-                                             State& o, State& d) {
-  double w[NS];
-  w[0] = h * k[0].scale;
-  constexpr int NI = FSAL ? NS - 1 : NS;  // stages whose input is a stage sum
+struct DormandPrince64 {
+  static constexpr int kStages = 7;
+  static constexpr bool kFsal = true;
+  static __device__ __forceinline__ double a(int s, int j) { return kDormandPrinceA[s][j]; }
+  static __device__ constexpr double b(int j) {
+    constexpr double B[7] = {dp::B1, 0, dp::B3, dp::B4, dp::B5, dp::B6, 0};
+    return B[j];
+  }
+  static __device__ constexpr double e(int j) {
+    constexpr double E[7] = {dp::D1, 0, dp::D3, dp::D4, dp::D5, dp::D6, dp::D7};
+    return E[j];
+  }
+};
+
+// One attempt. With have_first the first stage is `first`; otherwise it is
+// evaluated and returned there. `last` receives the last stage.
+//
+// The stage loop is rolled, with the stage values in local memory (~100
+// 8-byte loads per attempt, from L1): one copy of the evaluation keeps the
+// loop inside the instruction cache, where six copies with the products on
+// the integer pipes do not fit (the q-metric's least of all).
+template <class Met, class Tab, class A>
+__device__ __forceinline__ void rk_attempt64(const RayK& K, const State& y, double h,
+                                             bool have_first, Deriv& first, State& o, State& d,
+                                             Deriv& last, A& ar) {
+  constexpr int NS = Tab::kStages;
+  constexpr int NI = Tab::kFsal ? NS - 1 : NS;  // stages whose input is a stage sum
+  struct {
+    double r, th, ph, pr, pth, w;  // k~_j and w_j = h scale_j
+  } k[NS];
+  ar.window(h);
+  if (have_first) {
+    // a kept first stage may come from an attempt with plain instructions
+    if (!Met::kUnitScale) ar.window(first.scale);
+    k[0] = {first.r, first.th, first.ph, first.pr, first.pth,
+            Met::kUnitScale ? h : ar.soft(h, first.scale)};
+  }
+  auto fifth_order = [&]() {
+    o = y;
 #pragma unroll
-  for (int s = 1; s < NI; ++s) {
+    for (int j = 0; j < NI; ++j) {
+      if (Tab::b(j) != 0.0) {
+        const double c = ar.soft(Tab::b(j), k[j].w);
+        o.r = fma(c, k[j].r, o.r);
+        o.th = fma(c, k[j].th, o.th);
+        o.ph = fma(c, k[j].ph, o.ph);
+        o.pr = fma(c, k[j].pr, o.pr);
+        o.pth = fma(c, k[j].pth, o.pth);
+      }
+    }
+  };
+#pragma unroll 1
+  for (int s = have_first ? 1 : 0; s < NS; ++s) {
     double ir = y.r, it = y.th, ip = y.pr, iq = y.pth;
-#pragma unroll
-    for (int j = 0; j < s; ++j) {
-      if (T.a[s][j] != 0.0) {
-        const double c = T.a[s][j] * w[j];
+    if (Tab::kFsal && s == NS - 1) {
+      fifth_order();
+      ir = o.r;
+      it = o.th;
+      ip = o.pr;
+      iq = o.pth;
+    } else {
+#pragma unroll 1
+      for (int j = 0; j < s; ++j) {
+        const double c = ar.soft(Tab::a(s, j), k[j].w);
         ir = fma(c, k[j].r, ir);
         it = fma(c, k[j].th, it);
         ip = fma(c, k[j].pr, ip);
         iq = fma(c, k[j].pth, iq);
       }
     }
-    rhs64_at<Met>(K, ir, it, ip, iq, k[s]);
-    w[s] = h * k[s].scale;
+    Deriv ks;
+    rhs64_at<Met>(K, ir, it, ip, iq, ks, ar);
+    k[s] = {ks.r, ks.th, ks.ph, ks.pr, ks.pth, Met::kUnitScale ? h : ar.soft(h, ks.scale)};
+    if (s == 0) first = ks;
+    if (s == NS - 1) last = ks;
   }
-  o = y;
-#pragma unroll
-  for (int j = 0; j < NI; ++j) {
-    if (T.b[j] != 0.0) {
-      const double c = T.b[j] * w[j];
-      o.r = fma(c, k[j].r, o.r);
-      o.th = fma(c, k[j].th, o.th);
-      o.ph = fma(c, k[j].ph, o.ph);
-      o.pr = fma(c, k[j].pr, o.pr);
-      o.pth = fma(c, k[j].pth, o.pth);
-    }
-  }
-  if (FSAL) {
-    rhs64_at<Met>(K, o, k[NS - 1]);
-    w[NS - 1] = h * k[NS - 1].scale;
-  }
-  const double c0 = T.e[0] * w[0];
-  d.r = c0 * k[0].r;
-  d.th = c0 * k[0].th;
-  d.ph = c0 * k[0].ph;
-  d.pr = c0 * k[0].pr;
-  d.pth = c0 * k[0].pth;
+  if (!Tab::kFsal) fifth_order();
+  const double c0 = ar.soft(Tab::e(0), k[0].w);
+  d.r = ar.mul(c0, k[0].r);
+  d.th = ar.mul(c0, k[0].th);
+  d.ph = ar.mul(c0, k[0].ph);
+  d.pr = ar.mul(c0, k[0].pr);
+  d.pth = ar.mul(c0, k[0].pth);
 #pragma unroll
   for (int j = 1; j < NS; ++j) {
-    if (T.e[j] != 0.0) {
-      const double c = T.e[j] * w[j];
+    if (Tab::e(j) != 0.0) {
+      const double c = ar.soft(Tab::e(j), k[j].w);
       d.r = fma(c, k[j].r, d.r);
       d.th = fma(c, k[j].th, d.th);
       d.ph = fma(c, k[j].ph, d.ph);
@@ -509,44 +629,30 @@ __device__ __forceinline__ void rk_attempt64(const Tableau64<NS>& T, const RayK&
 }
 
 // One Cash-Karp attempt of length h from y (Sec. 3.1, RKCK45).
-template <class Met = KerrMetric>
+template <class Met = KerrMetric, class A = ArithPlain>
 __device__ __forceinline__ void ck_step64(const RayK& K, const State& y, double h, State& o,
-                                          State& d, double& twoH) {
-  constexpr Tableau64<6> T = {
-      {{0, 0, 0, 0, 0, 0},
-       {ck::A21, 0, 0, 0, 0, 0},
-       {ck::A31, ck::A32, 0, 0, 0, 0},
-       {ck::A41, ck::A42, ck::A43, 0, 0, 0},
-       {ck::A51, ck::A52, ck::A53, ck::A54, 0, 0},
-       {ck::A61, ck::A62, ck::A63, ck::A64, ck::A65, 0}},
-      {ck::B1, 0, ck::B3, ck::B4, 0, ck::B6},
-      {ck::D1, 0, ck::D3, ck::D4, ck::D5, ck::D6}};
-  Deriv k[6];
-  rhs64_at<Met>(K, y, k[0]);
-  twoH = k[0].twoH;
-  rk_attempt64<Met, 6, false>(T, K, y, h, k, o, d);
+                                          State& d, double& twoH, A&& ar = A()) {
+  Deriv first, last;
+  rk_attempt64<Met, CashKarp64>(K, y, h, false, first, o, d, last, ar);
+  twoH = first.twoH;
 }
 
-// One Dormand-Prince attempt of length h from y given k1 = f(y) (Sec. 3.1,
-// RKDP45): six new evaluations; k7 = f(o) is the first stage of the next
-// step if this one is accepted.
+// One Dormand-Prince attempt of length h from y (Sec. 3.1, RKDP45): k1 = f(y)
+// is given, or evaluated first and returned (have_first = false), then six
+// new evaluations; k7 = f(o) is the first stage of the next step if this one
+// is accepted.
+template <class Met = KerrMetric, class A = ArithPlain>
+__device__ __forceinline__ void dp_step64(const RayK& K, const State& y, double h,
+                                          bool have_first, Deriv& k1, State& o, State& d,
+                                          Deriv& k7, A&& ar = A()) {
+  rk_attempt64<Met, DormandPrince64>(K, y, h, have_first, k1, o, d, k7, ar);
+}
+
 template <class Met = KerrMetric>
 __device__ __forceinline__ void dp_step64(const RayK& K, const State& y, double h,
                                           const Deriv& k1, State& o, State& d, Deriv& k7) {
-  constexpr Tableau64<7> T = {
-      {{0, 0, 0, 0, 0, 0, 0},
-       {dp::A21, 0, 0, 0, 0, 0, 0},
-       {dp::A31, dp::A32, 0, 0, 0, 0, 0},
-       {dp::A41, dp::A42, dp::A43, 0, 0, 0, 0},
-       {dp::A51, dp::A52, dp::A53, dp::A54, 0, 0, 0},
-       {dp::A61, dp::A62, dp::A63, dp::A64, dp::A65, 0, 0},
-       {0, 0, 0, 0, 0, 0, 0}},  // the seventh stage is evaluated at o
-      {dp::B1, 0, dp::B3, dp::B4, dp::B5, dp::B6, 0},
-      {dp::D1, 0, dp::D3, dp::D4, dp::D5, dp::D6, dp::D7}};
-  Deriv k[7];
-  k[0] = k1;
-  rk_attempt64<Met, 7, true>(T, K, y, h, k, o, d);
-  k7 = k[6];
+  Deriv first = k1;
+  dp_step64<Met>(K, y, h, true, first, o, d, k7);
 }
 
 // True when x is +-inf or NaN (exponent bits all set); integer test only.
@@ -610,10 +716,25 @@ __device__ __forceinline__ double surface_value(int kind, const State& s, double
   return s.r - r_esc;
 }
 
+// a < b for b > 0 and an a that is not NaN, on the integer pipe.
+__device__ __forceinline__ bool less_than_positive(double a, double b) {
+  return bits_of(a) < bits_of(b);
+}
+
+// The smaller of two values that are not NaN, on the integer pipe: the bits
+// of a negative double order backwards, so all but its sign are flipped.
+__device__ __forceinline__ double min_by_bits(double a, double b) {
+  const long long ia = bits_of(a), ib = bits_of(b);
+  const long long ka = ia ^ ((ia >> 63) & 0x7fffffffffffffffLL);
+  const long long kb = ib ^ ((ib >> 63) & 0x7fffffffffffffffLL);
+  return kb < ka ? b : a;
+}
+
+// The sign of cos(theta) changes between two finite states. theta is a double
+// and pi/2 is not, so (PIO2_HI - theta) + PIO2_LO is never zero and is
+// positive exactly for theta <= PIO2_HI.
 __device__ __forceinline__ bool crosses_equator(const State& y0, const State& y1) {
-  const double c0 = (PIO2_HI - y0.th) + PIO2_LO;
-  const double c1 = (PIO2_HI - y1.th) + PIO2_LO;
-  return (c0 > 0.0 && c1 <= 0.0) || (c0 < 0.0 && c1 >= 0.0);
+  return (bits_of(y0.th) <= bits_of(PIO2_HI)) != (bits_of(y1.th) <= bits_of(PIO2_HI));
 }
 
 __device__ __forceinline__ const ReqDev* request_of(const KernelArgs& A, int k) {

@@ -5,6 +5,35 @@
 
 namespace osiris_impl {
 
+// Attempts outside the range of ArithFast (arith64.cuh), with plain FP64
+// instructions. Out of line, and on copies of its arguments, so that the
+// attempt loop keeps its state in registers.
+template <class Met>
+struct CkArgs {
+  RayK K;
+  State y, o, d;
+  double h, twoH;
+};
+
+template <class Met>
+__device__ __noinline__ void ck_step_plain(CkArgs<Met>& a) {
+  ck_step64<Met>(a.K, a.y, a.h, a.o, a.d, a.twoH);
+}
+
+template <class Met>
+struct DpArgs {
+  RayK K;
+  State y, o, d;
+  Deriv k1, k7;
+  double h;
+  bool have_first;  // k1 = f(y) is given
+};
+
+template <class Met>
+__device__ __noinline__ void dp_step_plain(DpArgs<Met>& a) {
+  dp_step64<Met>(a.K, a.y, a.h, a.have_first, a.k1, a.o, a.d, a.k7);
+}
+
 template <int INTEG, class Met>
 struct StepperFP64;
 
@@ -21,8 +50,19 @@ struct StepperFP64<OSIRIS_RKCK45, Met> {
   static __device__ __forceinline__ void accepted(LaneCache&) {}
   static __device__ __forceinline__ bool attempt(const RayK& K, const RayCache&, LaneCache&,
                                                  const State& y, double h, State& o, State& d,
-                                                 double& twoH) {
-    ck_step64<Met>(K, y, h, o, d, twoH);
+                                                 double& twoH, double one, double nz) {
+    ArithFast ar(one, nz);
+    ck_step64<Met>(K, y, h, o, d, twoH, ar);
+    if (ar.bad()) {
+      CkArgs<Met> a;
+      a.K = K;
+      a.y = y;
+      a.h = h;
+      ck_step_plain<Met>(a);
+      o = a.o;
+      d = a.d;
+      twoH = a.twoH;
+    }
     return true;
   }
   static __device__ __forceinline__ double twoH(const RayK& K, const State& y) {
@@ -48,20 +88,30 @@ struct StepperFP64<OSIRIS_RKDP45, Met> {
   static __device__ __forceinline__ void accepted(LaneCache& c) { c.k1 = c.k7; }
   static __device__ __forceinline__ bool attempt(const RayK& K, const RayCache&, LaneCache& c,
                                                  const State& y, double h, State& o, State& d,
-                                                 double& twoH) {
-    if (!c.valid) {
-      rhs64_at<Met>(K, y, c.k1);
-      c.valid = true;
+                                                 double& twoH, double one, double nz) {
+    ArithFast ar(one, nz);
+    dp_step64<Met>(K, y, h, c.valid, c.k1, o, d, c.k7, ar);
+    if (ar.bad()) {
+      DpArgs<Met> a;
+      a.K = K;
+      a.y = y;
+      a.h = h;
+      a.k1 = c.k1;
+      a.have_first = c.valid;
+      dp_step_plain<Met>(a);
+      o = a.o;
+      d = a.d;
+      c.k1 = a.k1;
+      c.k7 = a.k7;
     }
+    c.valid = true;
     twoH = c.k1.twoH;
-    dp_step64<Met>(K, y, h, c.k1, o, d, c.k7);
     return true;
   }
   static __device__ __forceinline__ double twoH(const RayK& K, const State& y) {
     return twoH64<Met>(K, y);
   }
 };
-
 
 template <int INTEG, class Met>
 __global__ void __maxnreg__(Met::kMaxRegs) trace_fp64_plain(const __grid_constant__ KernelArgs A) {

@@ -279,6 +279,8 @@ __device__ __forceinline__ void trace_body(const KernelArgs& A) {
   const unsigned FULL = 0xffffffffu;
   if (Stepper::kTrigTable) trig_table_init();
   if (Stepper::kExpLogTable) explog_table_init();
+  fma_units_init();
+  const double one = fma_units().one, nz = fma_units().nz;
 
   int mode = MODE_IDLE;
   bool drained = !PERSISTENT;
@@ -357,9 +359,9 @@ __device__ __forceinline__ void trace_body(const KernelArgs& A) {
   // the step end o (in this order), else continue from o. `fresh`: the last
   // attempt was the accepted step itself (its end-stage values are current).
   auto after_accept = [&](double hs, const State& o, bool fresh) {
-    if (o.r < r_cap) {
+    if (less_than_positive(o.r, r_cap)) {
       begin_locate(SURF_CAPTURE, hs, o);
-    } else if (o.r > r_esc) {
+    } else if (bits_of(o.r) > bits_of(r_esc)) {
       begin_locate(SURF_ESCAPE, hs, o);
     } else {
       y = o;
@@ -394,10 +396,11 @@ __device__ __forceinline__ void trace_body(const KernelArgs& A) {
     if (!__any_sync(FULL, mode != MODE_IDLE || has_claim())) break;
     if (mode != MODE_INTEGRATE && mode != MODE_LOCATE) continue;
 
-    const double hs = (mode == MODE_LOCATE) ? h_try : fmin(h, 0.1 * y.r);
+    // (a ray with a non-finite r ends at this attempt whatever its length)
+    const double hs = (mode == MODE_LOCATE) ? h_try : min_by_bits(h, 0.1 * y.r);
     State o, d;
     double twoH;
-    const bool fp64_step = Stepper::attempt(K, RC, LC, y, hs, o, d, twoH);
+    const bool fp64_step = Stepper::attempt(K, RC, LC, y, hs, o, d, twoH, one, nz);
     S.rhs += 6;
     S.fp64_steps += fp64_step ? 1 : 0;
 
