@@ -24,9 +24,9 @@
 // value), from which the range of every product follows; an attempt that
 // fails the test (bad()) is done again with plain FP64 instructions. Factors
 // that are zero in ordinary use (the spin of Schwarzschild, L of the middle
-// column, p_theta of the middle row) are never given to soft_mul.
+// column, p_theta of the middle row) are never given to soft_mul; those that a
+// soft_mul0 takes are tested with window0().
 #pragma once
-
 #include <cstdint>
 
 #include "convert.cuh"
@@ -81,17 +81,98 @@ __device__ __forceinline__ double soft_mul(double a, double b) {
 #endif
 }
 
+// soft_mul for an `a` that may also be zero (a product of zero keeps the sign
+// of the factors'). Four integer instructions more.
+__device__ __forceinline__ double soft_mul0(double a, double b) {
+  const double r = soft_mul(a, b);
+  const long long sign = (bits_of(a) ^ bits_of(b)) & (long long)0x8000000000000000ull;
+  const bool zero = ((unsigned)(bits_of(a) >> 32) & 0x7ff00000u) == 0;
+  return zero ? double_of(sign) : r;
+}
+
+// z 2^(e - 1086) with the sign bit `sign`, rounded to nearest even; the
+// leading bit of z is bit 60, 61 or 62, and every bit below the result's last
+// that is dropped before z was formed is in its bit 0.
+__device__ __forceinline__ double round_sum(uint64_t z, unsigned e, unsigned sign) {
+  const unsigned zh = (unsigned)(z >> 32), zl = (unsigned)z;
+  const unsigned top = zh >> 29;               // 0: bit 60, 1: bit 61, 2 or 3: bit 62
+  const unsigned n = 8 + (top > 2 ? 2 : top);  // bits dropped
+  const unsigned q2 = shift_r(zl, zh, n), q3 = zh >> n, q1 = shift_r(0u, zl, n);
+  const unsigned x = (q2 & 1u) + 0x7fffffffu;
+  const unsigned hi = q3 + ((e + n - 11u) << 20) + sign;  // the leading bit adds one to e
+#ifdef __CUDA_ARCH__
+  unsigned r2, r3;
+  asm("{\n\t.reg .u32 t;\n\tadd.cc.u32 t, %2, %3;\n\taddc.cc.u32 %0, %4, 0;\n\t"
+      "addc.u32 %1, %5, 0;\n\t}"
+      : "=r"(r2), "=r"(r3)
+      : "r"(q1), "r"(x), "r"(q2), "r"(hi));
+  return __hiloint2double((int)r3, (int)r2);
+#else
+  const uint64_t carry = ((uint64_t)q1 + x) >> 32;
+  return double_of((long long)((((uint64_t)hi << 32) | q2) + carry));
+#endif
+}
+
+// s + f, rounded to nearest even, for a normal s and a float f with |f| <
+// 2^-10 |s| (f zero or an FP32 denormal: s).
+__device__ __forceinline__ double soft_add_small(double s, float f) {
+  const unsigned sh = (unsigned)(bits_of(s) >> 32), sl = (unsigned)bits_of(s);
+  const unsigned fb = __float_as_uint(f);
+  const unsigned e = (sh >> 20) & 0x7ffu, ef = (fb >> 23) & 0xffu;
+  // significands with the leading bit at bit 61: s, and f shifted right by
+  // the difference d of the exponents; its bits beyond the last go into bit 0
+  const unsigned d0 = e - 896u - ef, d = d0 > 63u ? 63u : d0;
+  const unsigned m = ef ? (fb & 0x7fffffu) | 0x800000u : 0u;
+  const uint64_t x = ((uint64_t)((sh & 0xfffffu) | 0x100000u) << 41) | ((uint64_t)sl << 9);
+  const uint64_t v = (uint64_t)m << 38;
+  uint64_t y = v >> d;
+  if ((y << d) != v) y |= 1;
+  const uint64_t flip = (uint64_t)((long long)(int)(sh ^ fb) >> 63);
+  const uint64_t z = x + ((y ^ flip) - flip);
+  return round_sum(z, e + 1u, sh & 0x80000000u);
+}
+
+// x 2^k for an x of at most 53 significant bits and a normal result (or 0).
+__device__ __forceinline__ double exact_of(long long x, int k) {
+  const uint64_t u = (uint64_t)(x < 0 ? -x : x);
+  if (u == 0) return 0.0;
+  const int lz = clz64((long long)u);
+  const uint64_t m = (u << lz) >> 11;  // the leading bit at bit 52 adds one to the exponent
+  return double_of((long long)(((uint64_t)(x < 0) << 63) +
+                               ((uint64_t)(1085 - lz + k) << 52) + m));
+}
+
 // Plain FP64 instructions: the end point of a ray, and the attempts that
 // ArithFast gives back.
 struct ArithPlain {
   __device__ __forceinline__ double mul(double a, double b) const { return a * b; }
   __device__ __forceinline__ double soft(double a, double b) const { return a * b; }
+  __device__ __forceinline__ double soft0(double a, double b) const { return a * b; }
   __device__ __forceinline__ double add(double a, double c) const { return a + c; }
   __device__ __forceinline__ double sub(double a, double c) const { return a - c; }
   __device__ __forceinline__ double unit() const { return 1.0; }
+  // s + f for a correction f
+  __device__ __forceinline__ double add_small(double s, float f) const {
+    return s + float_to_double0(f);
+  }
+  __device__ __forceinline__ double minus_two(double r) const { return r - 2.0; }
   __device__ __forceinline__ void window(double) const {}
+  __device__ __forceinline__ void window0(double) const {}
 };
 
+// a + c on the FP64 unit where a sum on the integer pipes does not apply. Out
+// of line: the compiler would otherwise issue it every time and select.
+#ifdef __CUDACC__
+static __device__ __noinline__ double rare_add(double a, double c) { return a + c; }
+#else
+static inline double rare_add(double a, double c) { return a + c; }
+#endif
+
+// kSums: the sums that are cheap on the integer pipes go there too. That
+// takes 36 of an attempt's ~280 FP64 instructions, and makes its chain of
+// dependent instructions longer: worth it where enough warps are in flight to
+// hide that (kLargeLaunch in trace_fp64.cu).
+template <bool kSums>
 struct ArithFast {
   double one, nz;
   unsigned range;  // collects the exponent bits that leave the window
@@ -103,11 +184,34 @@ struct ArithFast {
   __device__ __forceinline__ double add(double a, double c) const { return fma(a, one, c); }
   __device__ __forceinline__ double sub(double a, double c) const { return fma(a, one, -c); }
   __device__ __forceinline__ double unit() const { return one; }
+  // Sums on the integer pipes where they are cheap there: a small correction,
+  // and differences that are exact (r - 2 is a multiple of the last place of r
+  // and no larger than r, so it is a double). Outside their range: native.
+  __device__ __forceinline__ double add_small(double s, float f) const {
+    if (!kSums) return add(s, float_to_double0(f));
+    const int d = (int)(((unsigned)(bits_of(s) >> 52)) & 0x7ffu) - 896 -
+                  (int)((__float_as_uint(f) >> 23) & 0xffu);
+    if (d < 11) return rare_add(s, float_to_double0(f));
+    return soft_add_small(s, f);
+  }
+  __device__ __forceinline__ double minus_two(double r) const {
+    if (!kSums) return sub(r, 2.0);
+    const unsigned shift = (unsigned)(bits_of(r) >> 52) - 1023u;  // r in [2^shift, 2^(shift+1))
+    if (shift > 52u) return rare_add(r, -2.0);
+    const long long m = (bits_of(r) & 0xfffffffffffffll) | 0x10000000000000ll;
+    return exact_of(m - (long long)(1ull << (53u - shift)), (int)shift - 52);
+  }
   // products on the integer pipes
   __device__ __forceinline__ double soft(double a, double b) const { return soft_mul(a, b); }
+  __device__ __forceinline__ double soft0(double a, double b) const { return soft_mul0(a, b); }
   // |x| in [2^-63, 2^65): biased exponents 960..1087, so that 64 more have the leading bits 1000
   __device__ __forceinline__ void window(double x) {
     range |= ((unsigned)(bits_of(x) >> 32) + 0x04000000u) ^ 0x40000000u;
+  }
+  // the same, or zero
+  __device__ __forceinline__ void window0(double x) {
+    const unsigned v = ((unsigned)(bits_of(x) >> 32) + 0x04000000u) ^ 0x40000000u;
+    range |= (bits_of(x) << 1) == 0 ? 0u : v;
   }
   __device__ __forceinline__ bool bad() const { return (range & 0x78000000u) != 0; }
 };

@@ -144,30 +144,32 @@ int sm_count(int* n) {
   return OSIRIS_OK;
 }
 
-using Launcher = int (*)(const KernelArgs&, Kernel, int, int, int, void*);
-
-Launcher launcher_of(const osiris_trace_opts* o) {
-  return (o->precision == OSIRIS_MIXED)  ? osiris_impl::launch_trace_mixed
-         : (o->precision == OSIRIS_DF64) ? osiris_impl::launch_trace_df64
-                                         : osiris_impl::launch_trace_fp64;
+const void* kernel_of(const osiris_trace_opts* o, Kernel kind, int spacetime, int64_t rays) {
+  const auto select = (o->precision == OSIRIS_MIXED)  ? osiris_impl::trace_kernel_mixed
+                      : (o->precision == OSIRIS_DF64) ? osiris_impl::trace_kernel_df64
+                                                      : osiris_impl::trace_kernel_fp64;
+  return select(kind, o->integrator, spacetime, rays);
 }
 
-// Launch shape of a persistent grid: threads per block and the full grid
-// (SMs x resident blocks per SM of the kernel that will run).
-int persistent_shape(const osiris_trace_opts* o, int spacetime, int* block,
-                     int64_t* full_grid) {
-  *block = o->block_size ? o->block_size : kDefaultBlock;
+int launch_kernel(const void* fn, const KernelArgs& args, int64_t grid, int block,
+                  cudaStream_t stream) {
+  void* params[] = {const_cast<KernelArgs*>(&args)};
+  return cuda_rc((int)cudaLaunchKernel(fn, dim3((unsigned)grid), dim3((unsigned)block), params, 0,
+                                       stream));
+}
+
+int block_of(const osiris_trace_opts* o) { return o->block_size ? o->block_size : kDefaultBlock; }
+
+// Blocks of a full persistent grid: SMs x resident blocks per SM of the kernel.
+int full_grid(const osiris_trace_opts* o, const void* fn, int64_t* grid) {
   int sms = 0;
   if (int rc = sm_count(&sms)) return rc;
   int per_sm = o->blocks_per_sm;
-  if (per_sm == 0) {
-    auto occ = (o->precision == OSIRIS_MIXED)  ? osiris_impl::occupancy_mixed
-               : (o->precision == OSIRIS_DF64) ? osiris_impl::occupancy_df64
-                                               : osiris_impl::occupancy_fp64;
-    if (occ(Kernel::kPersistent, o->integrator, spacetime, *block, &per_sm) != 0 || per_sm < 1)
-      return OSIRIS_ECUDA;
-  }
-  *full_grid = static_cast<int64_t>(sms) * per_sm;
+  if (per_sm == 0 &&
+      (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, block_of(o), 0) != cudaSuccess ||
+       per_sm < 1))
+    return OSIRIS_ECUDA;
+  *grid = static_cast<int64_t>(sms) * per_sm;
   return OSIRIS_OK;
 }
 
@@ -197,31 +199,27 @@ void set_granularity(KernelArgs& args, const osiris_trace_opts* o) {
 int launch(KernelArgs& args, const osiris_trace_opts* o, void* stream) {
   if (args.total_rays == 0) return OSIRIS_OK;
   const bool persistent = o->persistent != 0 || args.reqs != nullptr;
-  const Launcher launcher = launcher_of(o);
-  set_granularity(args, o);
-  if (!persistent) {
-    const int block = o->block_size ? o->block_size : kDefaultBlock;
-    const int64_t per_block = static_cast<int64_t>(block) * args.rays_per_lane;
-    const int64_t grid = (args.total_rays + per_block - 1) / per_block;
-    if (grid > 0x7fffffff) return OSIRIS_EINVAL;
-    args.queue = nullptr;
-    return cuda_rc(
-        launcher(args, Kernel::kPlain, o->integrator, static_cast<int>(grid), block, stream));
-  }
-  if (!o->workspace || o->workspace_bytes < osiris_impl::kQueueBytes) return OSIRIS_ENOMEM;
-  int block = 0;
-  int64_t grid = 0;
   const int spacetime = args.reqs ? args.spacetime : args.single.spacetime;
-  if (int rc = persistent_shape(o, spacetime, &block, &grid)) return rc;
+  const int block = block_of(o);
+  cudaStream_t s = static_cast<cudaStream_t>(stream);
+  set_granularity(args, o);
   const int64_t per_block = static_cast<int64_t>(block) * args.rays_per_lane;
   const int64_t needed = (args.total_rays + per_block - 1) / per_block;
+  if (!persistent) {
+    if (needed > 0x7fffffff) return OSIRIS_EINVAL;
+    args.queue = nullptr;
+    return launch_kernel(kernel_of(o, Kernel::kPlain, spacetime, args.total_rays), args, needed,
+                         block, s);
+  }
+  if (!o->workspace || o->workspace_bytes < osiris_impl::kQueueBytes) return OSIRIS_ENOMEM;
+  const void* fn = kernel_of(o, Kernel::kPersistent, spacetime, args.total_rays);
+  int64_t grid = 0;
+  if (int rc = full_grid(o, fn, &grid)) return rc;
   if (grid > needed) grid = needed;
   args.queue = static_cast<unsigned long long*>(o->workspace);
-  cudaStream_t s = static_cast<cudaStream_t>(stream);
   if (cudaMemsetAsync(args.queue, 0, sizeof(unsigned long long), s) != cudaSuccess)
     return OSIRIS_ECUDA;
-  return cuda_rc(
-      launcher(args, Kernel::kPersistent, o->integrator, static_cast<int>(grid), block, stream));
+  return launch_kernel(fn, args, grid, block, s);
 }
 
 // Validate a batch and fill its request table (host memory, n entries);
@@ -646,7 +644,11 @@ struct osiris_batch_plan {
   int32_t max_requests = 0;
   int32_t spacetime = OSIRIS_SPACETIME_KERR;
   int block = 0;
-  int64_t full_grid = 0;
+  // the kernels of a small and of a large launch, each with its full grid
+  struct {
+    const void* fn;
+    int64_t full_grid;
+  } variant[2] = {};
   ReqDev* staging = nullptr;    // pinned host copy of the request table
   ReqDev* dev_table = nullptr;  // inside opts.workspace
   cudaEvent_t copied = nullptr;  // recorded by the graph once the table is uploaded
@@ -693,7 +695,7 @@ int record_plan(osiris_batch_plan* p) {
                       cudaMemcpyHostToDevice, cs) != cudaSuccess ||
       cudaEventRecordWithFlags(p->copied, cs, cudaEventRecordExternal) != cudaSuccess ||
       cudaMemsetAsync(args.queue, 0, sizeof(unsigned long long), cs) != cudaSuccess ||
-      launcher_of(&p->opts)(args, Kernel::kPersistent, p->opts.integrator, 1, p->block, cs) != 0)
+      launch_kernel(p->variant[0].fn, args, 1, p->block, cs) != OSIRIS_OK)
     rc = OSIRIS_ECUDA;
   cudaGraph_t g = nullptr;
   if (cudaStreamEndCapture(cs, &g) != cudaSuccess) rc = OSIRIS_ECUDA;
@@ -744,7 +746,12 @@ int osiris_batch_plan_create(osiris_batch_plan** out, int32_t max_requests, int3
   p->spacetime = spacetime;
   p->dev_table = reinterpret_cast<ReqDev*>(static_cast<char*>(opts->workspace) +
                                            osiris_impl::kQueueBytes);
-  int rc = persistent_shape(&p->opts, spacetime, &p->block, &p->full_grid);
+  p->block = block_of(&p->opts);
+  int rc = OSIRIS_OK;
+  for (int k = 0; k < 2 && rc == OSIRIS_OK; ++k) {
+    p->variant[k].fn = kernel_of(&p->opts, Kernel::kPersistent, spacetime, k ? INT64_MAX : 1);
+    rc = full_grid(&p->opts, p->variant[k].fn, &p->variant[k].full_grid);
+  }
   if (rc == OSIRIS_OK &&
       cudaMallocHost(&p->staging, sizeof(ReqDev) * static_cast<size_t>(max_requests)) !=
           cudaSuccess) {
@@ -788,8 +795,11 @@ int osiris_batch_plan_launch(osiris_batch_plan* p, const osiris_request* reqs, i
   set_granularity(args, &p->opts);
   const int64_t per_block = static_cast<int64_t>(p->block) * args.rays_per_lane;
   int64_t grid = (total + per_block - 1) / per_block;
-  if (grid > p->full_grid) grid = p->full_grid;
+  const void* fn = kernel_of(&p->opts, Kernel::kPersistent, p->spacetime, total);
+  const int64_t most = p->variant[fn == p->variant[0].fn ? 0 : 1].full_grid;
+  if (grid > most) grid = most;
   cudaKernelNodeParams k = p->kernel;
+  k.func = const_cast<void*>(fn);
   void* argv[] = {&args};
   k.gridDim = dim3(static_cast<unsigned>(grid), 1, 1);
   k.kernelParams = argv;

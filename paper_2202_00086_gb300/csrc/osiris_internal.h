@@ -64,17 +64,11 @@ constexpr size_t kQueueBytes = 256;  // workspace head: the ray counter
 
 enum class Kernel { kPlain, kPersistent };
 
-// Launchers implemented in the kernel translation units. They return a
-// cudaError_t value as int (0 = success).
-int launch_trace_fp64(const KernelArgs& args, Kernel kind, int integrator, int grid, int block,
-                      void* stream);
-int launch_trace_mixed(const KernelArgs& args, Kernel kind, int integrator, int grid, int block,
-                       void* stream);
-int launch_trace_df64(const KernelArgs& args, Kernel kind, int integrator, int grid, int block,
-                      void* stream);
-int occupancy_fp64(Kernel kind, int integrator, int spacetime, int block, int* blocks_per_sm);
-int occupancy_mixed(Kernel kind, int integrator, int spacetime, int block, int* blocks_per_sm);
-int occupancy_df64(Kernel kind, int integrator, int spacetime, int block, int* blocks_per_sm);
+// The trace kernel of a launch: by precision, kind, integrator, space-time and
+// the launch's rays.
+const void* trace_kernel_fp64(Kernel kind, int integrator, int spacetime, int64_t rays);
+const void* trace_kernel_mixed(Kernel kind, int integrator, int spacetime, int64_t rays);
+const void* trace_kernel_df64(Kernel kind, int integrator, int spacetime, int64_t rays);
 // Pipe probes (roofline denominators): 16 chains per thread of one
 // operation (0 FMA, 1 multiply, 2 add, 3 multiply as FMA, 4 add as FMA),
 // 256 threads per block.

@@ -123,7 +123,7 @@ constexpr int kTrigNodes = kTrigPerPi + 2 * (kTrigPerPi / 16) + 1;
 struct TrigTable {
   double2 sc[kTrigNodes];  // sin N_k, cos N_k
   float4 scf[kTrigNodes];  // the same as double-float pairs (sin hi, lo, cos hi, lo)
-  double n[kTrigNodes];    // N_k
+  uint64_t n62[kTrigNodes];  // N_k 2^62 (N_k >= 0)
 };
 
 __device__ __forceinline__ TrigTable& trig_table() {
@@ -131,18 +131,23 @@ __device__ __forceinline__ TrigTable& trig_table() {
   return table;
 }
 
+// N_k of table entry i: the double nearest to k pi/512.
+__device__ __forceinline__ double trig_node(int i) {
+  constexpr double STEP = 3.141592653589793116 / kTrigPerPi;  // exact: pi rounded / 2^9
+  return (double)(i + kTrigFirst) * STEP;
+}
+
 // Fill the block's table (all threads of the block, before any divergence).
 __device__ __forceinline__ void trig_table_init() {
-  constexpr double STEP = 3.141592653589793116 / kTrigPerPi;  // exact: pi rounded / 2^9
   TrigTable& t = trig_table();
   for (int i = threadIdx.x; i < kTrigNodes; i += blockDim.x) {
-    const double n = (double)(i + kTrigFirst) * STEP;
+    const double n = trig_node(i);
     double s, c;
     sincos(n, &s, &c);
     t.sc[i] = make_double2(s, c);
     const float sh = (float)s, ch = (float)c;
     t.scf[i] = make_float4(sh, (float)(s - (double)sh), ch, (float)(c - (double)ch));
-    t.n[i] = n;
+    t.n62[i] = n > 0.0 ? (uint64_t)(n * 0x1p62) : 0;
   }
   __syncthreads();
 }
@@ -221,6 +226,21 @@ __device__ __forceinline__ float add_as_fma(float a, float c) { return a + c; }
 
 
 
+// theta - N_k, exact. For theta in [2^-10, 4), where N_k and the last place of
+// theta are multiples of 2^-62, on the integer pipes.
+__device__ __forceinline__ double node_difference(double th, uint64_t, int i, const ArithPlain&) {
+  return th - trig_node(i);
+}
+template <bool kSums>
+__device__ __forceinline__ double node_difference(double th, uint64_t n62, int i,
+                                                  const ArithFast<kSums>& ar) {
+  if (!kSums) return ar.sub(th, trig_node(i));
+  const unsigned shift = (unsigned)((uint64_t)bits_of(th) >> 52) - 1013u;
+  if (shift > 11u) return rare_add(th, -trig_node(i));
+  const uint64_t m = ((uint64_t)bits_of(th) & 0xfffffffffffffull) | 0x10000000000000ull;
+  return exact_of((long long)((m << shift) - n62), -62);
+}
+
 template <class A = ArithPlain>
 __device__ __forceinline__ void sincos_tab(double th, double& s, double& c, A&& ar = A()) {
   using namespace dfc;
@@ -235,7 +255,7 @@ __device__ __forceinline__ void sincos_tab(double th, double& s, double& c, A&& 
   const TrigTable& t = trig_table();
   const double2 sc = t.sc[idx];
   const float4 scf = t.scf[idx];
-  const double x = ar.sub(th, t.n[idx]);  // exact
+  const double x = node_difference(th, t.n62[idx], idx, ar);  // exact
   // the corrections in double-float
   const df xd = split_df(x);
   const df u = df_sqr(xd);                                                    // x^2
@@ -246,10 +266,8 @@ __device__ __forceinline__ void sincos_tab(double th, double& s, double& c, A&& 
   const df S = mk(scf.x, scf.y), C = mk(scf.z, scf.w);
   const df corr_s = df_add_u(df_mul(C, ds), df_mul(S, cm));
   const df corr_c = df_sub_u(df_mul(C, cm), df_mul(S, ds));
-  s = ar.add(fma(sc.y, x, ar.add(sc.x, float_to_double0(corr_s.hi))),
-             float_to_double0(corr_s.lo));
-  c = ar.add(fma(-sc.x, x, ar.add(sc.y, float_to_double0(corr_c.hi))),
-             float_to_double0(corr_c.lo));
+  s = ar.add_small(fma(sc.y, x, ar.add_small(sc.x, corr_s.hi)), corr_s.lo);
+  c = ar.add_small(fma(-sc.x, x, ar.add_small(sc.y, corr_c.hi)), corr_c.lo);
 }
 
 // max |H - H0| kept as the bit pattern of a non-negative double: |v| and the
@@ -304,9 +322,8 @@ __device__ __forceinline__ double rcp64(double d, A&& ar = A()) {
 // Y = p_r^2 + u^2, L / sin reused). twoH receives 2H = N / Sigma at the
 // evaluation point.
 // ---------------------------------------------------------------------------
-// With ArithFast the products of factors that ordinary rays keep away from
-// zero go to the integer pipes; the others may vanish (a = 0, L = 0, cos = 0)
-// and stay on the FP64 unit.
+// With ArithFast every product goes to the integer pipes (those that vanish for
+// a = 0 or L = 0 through soft0; window_constants tests K once per attempt).
 template <class A = ArithPlain>
 __device__ __forceinline__ void rhs64(const RayK& K, double r, double th, double pr, double pth,
                                       double& dr, double& dth, double& dph, double& dpr,
@@ -314,8 +331,8 @@ __device__ __forceinline__ void rhs64(const RayK& K, double r, double th, double
   double s, c;
   sincos_tab(th, s, c, ar);
   const double ra2 = fma(r, r, K.a2);  // r^2 + a^2
-  const double a2s = ar.mul(K.a2, s);
-  const double Delta = fma(r, ar.sub(r, 2.0), K.a2);
+  const double a2s = ar.soft0(K.a2, s);
+  const double Delta = fma(r, ar.minus_two(r), K.a2);
   // Sigma = r^2 + a^2 cos^2 = (r^2 + a^2) - a^2 sin^2 (no cancellation: r > a)
   const double Sigma = fma(-a2s, s, ra2);
   const double P = fma(ra2, K.E, -K.aL);
@@ -330,7 +347,7 @@ __device__ __forceinline__ void rhs64(const RayK& K, double r, double th, double
   const double iSig = ar.soft(Delta, sinv);
   const double iDel = ar.soft(Sigma, sinv);
   const double is = ar.soft(DS, inv);
-  const double Lis = ar.mul(K.L, is);  // L / sin
+  const double Lis = ar.soft0(K.L, is);  // L / sin
   const double W = fma(-K.aE, s, Lis);
   const double u = ar.soft(P, iDel);
   const double Dpr = ar.soft(Delta, pr);
@@ -341,12 +358,15 @@ __device__ __forceinline__ void rhs64(const RayK& K, double r, double th, double
   // (scale) and folded into the stepper's tableau coefficients.
   dr = Dpr;
   dth = pth;
-  dph = fma(W, is, ar.mul(K.a, u));
+  dph = fma(W, is, ar.soft0(K.a, u));
   // -dH/dr: (1 - r) Y + r X = Y + r (X - Y), Y = u^2 + p_r^2, X = 2H + 2E u
   const double Y = fma(u, u, ar.soft(pr, pr));
   dpr = fma(r, ar.sub(fma(K.E2, u, NiS), Y), Y);
   // -dH/dtheta: cos (W (L / sin^2 + a E) - a^2 sin 2H)
-  dpth = ar.mul(c, fma(W, fma(Lis, is, K.aE), -ar.mul(a2s, NiS)));
+  const double F = fma(W, fma(Lis, is, K.aE), -ar.soft0(a2s, NiS));
+  ar.window(c);
+  ar.window0(F);
+  dpth = ar.soft0(F, c);
   scale = iSig;
   twoH = NiS;
 }
@@ -373,7 +393,7 @@ __device__ __forceinline__ void rhs_q64(const RayK& K, double r, double th, doub
   sincos_tab(th, s, c, ar);
   // four reciprocals (1/D, 1/X, 1/sin^2, 1/(f f^q)) serve every quotient:
   // 1/r = (r - 2)/D, and f = (r - 2)/r keeps its relative accuracy at r -> 2
-  const double rm2 = ar.sub(r, 2.0);
+  const double rm2 = ar.minus_two(r);
   ar.window(r);
   ar.window(rm2);
   ar.window(s);
@@ -424,19 +444,16 @@ __device__ __forceinline__ void rhs_q64(const RayK& K, double r, double th, doub
 }
 
 // Metric policies for the FP64 steppers.
-#ifndef OSIRIS_FP64_MAXREGS
-#define OSIRIS_FP64_MAXREGS 255
-#endif
-
 struct KerrMetric {
   static constexpr bool kTrigTable = true;  // rhs64 reads the block's sincos table
   static constexpr bool kExpLogTable = false;
-  // No register cap (the compiler takes ~200, two blocks of 128 threads per
-  // SM): measured on the 12 x 1024^2 Kerr set, 3.09 Mrays/s uncapped against
-  // 2.95 at 168 registers (three blocks) and 2.90 at 152 or 128 (three or
-  // four blocks). The FP64 pipe needs the scheduling freedom more than warps.
-  static constexpr int kMaxRegs = OSIRIS_FP64_MAXREGS;
   static constexpr bool kUnitScale = false;
+  template <class A>
+  static __device__ __forceinline__ void window_constants(const RayK& K, A& ar) {
+    ar.window0(K.a);
+    ar.window0(K.a2);
+    ar.window0(K.L);
+  }
   template <class A>
   static __device__ __forceinline__ void rhs(const RayK& K, double r, double th, double pr,
                                              double pth, double& dr, double& dth, double& dph,
@@ -448,8 +465,9 @@ struct KerrMetric {
 struct QMetric {
   static constexpr bool kTrigTable = true;  // rhs_q64 reads the block's sincos table
   static constexpr bool kExpLogTable = true;  // and the exp/log tables
-  static constexpr int kMaxRegs = OSIRIS_FP64_MAXREGS;
   static constexpr bool kUnitScale = true;
+  template <class A>
+  static __device__ __forceinline__ void window_constants(const RayK&, A&) {}
   template <class A>
   static __device__ __forceinline__ void rhs(const RayK& K, double r, double th, double pr,
                                              double pth, double& dr, double& dth, double& dph,
@@ -552,7 +570,10 @@ struct DormandPrince64 {
 // The stage loop is rolled, with the stage values in local memory (~100
 // 8-byte loads per attempt, from L1): one copy of the evaluation keeps the
 // loop inside the instruction cache, where six copies with the products on
-// the integer pipes do not fit (the q-metric's least of all).
+// the integer pipes do not fit (the q-metric's least of all). Measured with
+// plain FP64 multiplies and six copies / products on the integer pipes and
+// six copies / and one copy: twelve 320^2 Kerr renders in one launch 338 /
+// 267 / 248 ms, a 333 x 257 q-metric render 57.3 / 59.9 / 44.2 ms.
 template <class Met, class Tab, class A>
 __device__ __forceinline__ void rk_attempt64(const RayK& K, const State& y, double h,
                                              bool have_first, Deriv& first, State& o, State& d,
@@ -563,6 +584,7 @@ __device__ __forceinline__ void rk_attempt64(const RayK& K, const State& y, doub
     double r, th, ph, pr, pth, w;  // k~_j and w_j = h scale_j
   } k[NS];
   ar.window(h);
+  Met::window_constants(K, ar);
   if (have_first) {
     // a kept first stage may come from an attempt with plain instructions
     if (!Met::kUnitScale) ar.window(first.scale);

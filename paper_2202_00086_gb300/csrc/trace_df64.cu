@@ -105,22 +105,9 @@ static const void* df64_kernel(Kernel kind, int integrator) {
                                      : df64_kernel<Met, OSIRIS_RKCK45>(kind);
 }
 
-static const void* select_df64(Kernel kind, int integrator, int spacetime) {
+const void* trace_kernel_df64(Kernel kind, int integrator, int spacetime, int64_t) {
   return spacetime == OSIRIS_SPACETIME_QMETRIC ? df64_kernel<QMetricDF>(kind, integrator)
                                                : df64_kernel<KerrDF>(kind, integrator);
-}
-
-int launch_trace_df64(const KernelArgs& args, Kernel kind, int integrator, int grid, int block,
-                      void* stream) {
-  const int spacetime = args.reqs ? args.spacetime : args.single.spacetime;
-  void* params[] = {const_cast<KernelArgs*>(&args)};
-  return (int)cudaLaunchKernel(select_df64(kind, integrator, spacetime), dim3(grid),
-                               dim3(block), params, 0, static_cast<cudaStream_t>(stream));
-}
-
-int occupancy_df64(Kernel kind, int integrator, int spacetime, int block, int* blocks_per_sm) {
-  return (int)cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-      blocks_per_sm, select_df64(kind, integrator, spacetime), block, 0);
 }
 
 }  // namespace osiris_impl

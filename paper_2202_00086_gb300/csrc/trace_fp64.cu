@@ -34,12 +34,12 @@ __device__ __noinline__ void dp_step_plain(DpArgs<Met>& a) {
   dp_step64<Met>(a.K, a.y, a.h, a.have_first, a.k1, a.o, a.d, a.k7);
 }
 
-template <int INTEG, class Met>
+template <int INTEG, class Met, bool kLarge>
 struct StepperFP64;
 
 // Cash-Karp: every attempt evaluates its six stages.
-template <class Met>
-struct StepperFP64<OSIRIS_RKCK45, Met> {
+template <class Met, bool kLarge>
+struct StepperFP64<OSIRIS_RKCK45, Met, kLarge> {
   static constexpr double kLocateRel = 0.0;
   static constexpr bool kTrigTable = Met::kTrigTable;
   static constexpr bool kExpLogTable = Met::kExpLogTable;
@@ -51,7 +51,7 @@ struct StepperFP64<OSIRIS_RKCK45, Met> {
   static __device__ __forceinline__ bool attempt(const RayK& K, const RayCache&, LaneCache&,
                                                  const State& y, double h, State& o, State& d,
                                                  double& twoH, double one, double nz) {
-    ArithFast ar(one, nz);
+    ArithFast<kLarge> ar(one, nz);
     ck_step64<Met>(K, y, h, o, d, twoH, ar);
     if (ar.bad()) {
       CkArgs<Met> a;
@@ -73,8 +73,8 @@ struct StepperFP64<OSIRIS_RKCK45, Met> {
 // Dormand-Prince: k1 is carried from the previous accepted attempt's seventh
 // stage; it is evaluated only when a ray starts or resumes (a warp evaluates
 // it when any of its lanes needs it).
-template <class Met>
-struct StepperFP64<OSIRIS_RKDP45, Met> {
+template <class Met, bool kLarge>
+struct StepperFP64<OSIRIS_RKDP45, Met, kLarge> {
   static constexpr double kLocateRel = 0.0;
   static constexpr bool kTrigTable = Met::kTrigTable;
   static constexpr bool kExpLogTable = Met::kExpLogTable;
@@ -89,7 +89,7 @@ struct StepperFP64<OSIRIS_RKDP45, Met> {
   static __device__ __forceinline__ bool attempt(const RayK& K, const RayCache&, LaneCache& c,
                                                  const State& y, double h, State& o, State& d,
                                                  double& twoH, double one, double nz) {
-    ArithFast ar(one, nz);
+    ArithFast<kLarge> ar(one, nz);
     dp_step64<Met>(K, y, h, c.valid, c.k1, o, d, c.k7, ar);
     if (ar.bad()) {
       DpArgs<Met> a;
@@ -113,42 +113,53 @@ struct StepperFP64<OSIRIS_RKDP45, Met> {
   }
 };
 
-template <int INTEG, class Met>
-__global__ void __maxnreg__(Met::kMaxRegs) trace_fp64_plain(const __grid_constant__ KernelArgs A) {
-  trace_body<StepperFP64<INTEG, Met>, false>(A);
+// Two variants of the Kerr kernels, chosen by the launch's rays.
+//
+// Small launches last as long as their slowest warps' chains of dependent
+// instructions: sums on the FP64 unit, no register cap (the compiler takes
+// ~195, two blocks of 128 threads per SM). Large ones are bound by the FP64
+// unit: sums on the integer pipes where they are cheap there (ArithFast<true>),
+// and four blocks per SM to hide the longer chains. Small / large variant, ms:
+//   Cash-Karp   render    64^2  13.7 / 16.2     320^2  32.8 / 31.8
+//                        384^2  44.1 / 42.9     512^2  64.4 / 58.9
+//                        768^2   131 / 110      twelve 400^2 in a batch 382 / 347
+//   particles  30,000     2.7 / 2.9             500,000  33.8 / 30.0
+//   Dormand-Prince disk  512 x 256  30.0 / 33.4     600 x 300  35.0 / 35.0
+//                        800 x 400  56.2 / 54.1    1024 x 512  89.3 / 80.2
+// The line lies at five times the lanes that the small variant keeps in
+// flight. Caps of 168 registers (three blocks) with either sums lie between
+// the two. The q-metric has the small variant only: twice the integer work
+// per evaluation, and the large one is 1-5 % slower up to six 400^2 renders.
+constexpr int64_t kLargeLaunch = 5 * 152 * 256;
+
+template <int INTEG, class Met, bool kLarge>
+__global__ void __maxnreg__(kLarge ? 128 : 255)
+    trace_fp64_plain(const __grid_constant__ KernelArgs A) {
+  trace_body<StepperFP64<INTEG, Met, kLarge>, false>(A);
 }
 
-template <int INTEG, class Met>
-__global__ void __maxnreg__(Met::kMaxRegs) trace_fp64_persistent(const __grid_constant__ KernelArgs A) {
-  trace_body<StepperFP64<INTEG, Met>, true>(A);
+template <int INTEG, class Met, bool kLarge>
+__global__ void __maxnreg__(kLarge ? 128 : 255)
+    trace_fp64_persistent(const __grid_constant__ KernelArgs A) {
+  trace_body<StepperFP64<INTEG, Met, kLarge>, true>(A);
 }
 
-template <int INTEG, class Met>
+template <int INTEG, class Met, bool kLarge>
 static const void* fp64_kernel(Kernel kind) {
-  return kind == Kernel::kPersistent ? (const void*)trace_fp64_persistent<INTEG, Met>
-                                     : (const void*)trace_fp64_plain<INTEG, Met>;
+  return kind == Kernel::kPersistent ? (const void*)trace_fp64_persistent<INTEG, Met, kLarge>
+                                     : (const void*)trace_fp64_plain<INTEG, Met, kLarge>;
 }
 
-static const void* select_fp64(Kernel kind, int integrator, int spacetime) {
-  if (spacetime == OSIRIS_SPACETIME_QMETRIC)
-    return integrator == OSIRIS_RKDP45 ? fp64_kernel<OSIRIS_RKDP45, QMetric>(kind)
-                                       : fp64_kernel<OSIRIS_RKCK45, QMetric>(kind);
-  return integrator == OSIRIS_RKDP45 ? fp64_kernel<OSIRIS_RKDP45, KerrMetric>(kind)
-                                     : fp64_kernel<OSIRIS_RKCK45, KerrMetric>(kind);
+template <class Met, bool kLarge>
+static const void* fp64_kernel(Kernel kind, int integrator) {
+  return integrator == OSIRIS_RKDP45 ? fp64_kernel<OSIRIS_RKDP45, Met, kLarge>(kind)
+                                     : fp64_kernel<OSIRIS_RKCK45, Met, kLarge>(kind);
 }
 
-int launch_trace_fp64(const KernelArgs& args, Kernel kind, int integrator, int grid, int block,
-                      void* stream) {
-  const int spacetime = args.reqs ? args.spacetime : args.single.spacetime;
-  const void* fn = select_fp64(kind, integrator, spacetime);
-  void* params[] = {const_cast<KernelArgs*>(&args)};
-  return (int)cudaLaunchKernel(fn, dim3(grid), dim3(block), params, 0,
-                               static_cast<cudaStream_t>(stream));
-}
-
-int occupancy_fp64(Kernel kind, int integrator, int spacetime, int block, int* blocks_per_sm) {
-  return (int)cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-      blocks_per_sm, select_fp64(kind, integrator, spacetime), block, 0);
+const void* trace_kernel_fp64(Kernel kind, int integrator, int spacetime, int64_t rays) {
+  if (spacetime == OSIRIS_SPACETIME_QMETRIC) return fp64_kernel<QMetric, false>(kind, integrator);
+  return rays >= kLargeLaunch ? fp64_kernel<KerrMetric, true>(kind, integrator)
+                              : fp64_kernel<KerrMetric, false>(kind, integrator);
 }
 
 // Roofline probes: kProbeChains independent chains of one arithmetic

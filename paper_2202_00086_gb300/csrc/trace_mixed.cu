@@ -143,22 +143,9 @@ static const void* mixed_kernel(Kernel kind, int integrator) {
                                      : mixed_kernel<Met, OSIRIS_RKCK45>(kind);
 }
 
-static const void* select_mixed(Kernel kind, int integrator, int spacetime) {
+const void* trace_kernel_mixed(Kernel kind, int integrator, int spacetime, int64_t) {
   return spacetime == OSIRIS_SPACETIME_QMETRIC ? mixed_kernel<QMetricMixed>(kind, integrator)
                                                : mixed_kernel<KerrMixed>(kind, integrator);
-}
-
-int launch_trace_mixed(const KernelArgs& args, Kernel kind, int integrator, int grid, int block,
-                       void* stream) {
-  const int spacetime = args.reqs ? args.spacetime : args.single.spacetime;
-  void* params[] = {const_cast<KernelArgs*>(&args)};
-  return (int)cudaLaunchKernel(select_mixed(kind, integrator, spacetime), dim3(grid),
-                               dim3(block), params, 0, static_cast<cudaStream_t>(stream));
-}
-
-int occupancy_mixed(Kernel kind, int integrator, int spacetime, int block, int* blocks_per_sm) {
-  return (int)cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-      blocks_per_sm, select_mixed(kind, integrator, spacetime), block, 0);
 }
 
 }  // namespace osiris_impl

@@ -3,6 +3,7 @@ as host C++, against plain FP64 operations, bit for bit:
   - soft_mul over the exponents its callers admit, with dense significands,
     significands of a few bits and products exactly halfway between two
     doubles;
+  - the sums with a small correction and the exact r - 2;
   - whole Cash-Karp and Dormand-Prince attempts, Kerr and the q-metric, with
     ArithFast against the same attempt with ArithPlain: equal wherever
     ArithFast does not give the attempt back, which it does not for ordinary
@@ -19,7 +20,7 @@ from _df_host import build
 HARNESS = r"""
 #include "trace_device.cuh"
 using namespace osiris_impl;
-template <class Met>
+template <class Met, bool kSums>
 static void attempt(const double* in, double* out) {
   RayK K;
   K.a = in[2];
@@ -41,7 +42,7 @@ static void attempt(const double* in, double* out) {
   State o[2], d[2];
   Deriv k1[2] = {}, k7[2] = {};
   double twoH[2];
-  ArithFast fast(1.0, -0.0);
+  ArithFast<kSums> fast(1.0, -0.0);
   if (in[1] == 0.0) {
     ck_step64<Met>(K, y, h, o[0], d[0], twoH[0], fast);
     ck_step64<Met>(K, y, h, o[1], d[1], twoH[1]);
@@ -69,11 +70,20 @@ int main(int, char** argv) {
     }
     return 0;
   }
+  if (argv[1][0] == 'a') {  // s, f: s + f, and f - 2 as a double
+    while (std::fread(in, sizeof(double), 2, stdin) == 2) {
+      ArithFast<true> fast(1.0, -0.0);
+      out[0] = fast.add_small(in[0], (float)in[1]);
+      out[1] = fast.minus_two(std::fabs(in[0]));
+      std::fwrite(out, sizeof(double), 2, stdout);
+    }
+    return 0;
+  }
   while (std::fread(in, sizeof(double), 11, stdin) == 11) {
-    if (in[0] == 0.0)
-      attempt<KerrMetric>(in, out);
+    if (argv[1][0] == 's')
+      in[0] == 0.0 ? attempt<KerrMetric, true>(in, out) : attempt<QMetric, true>(in, out);
     else
-      attempt<QMetric>(in, out);
+      in[0] == 0.0 ? attempt<KerrMetric, false>(in, out) : attempt<QMetric, false>(in, out);
     std::fwrite(out, sizeof(double), 23, stdout);
   }
   return 0;
@@ -136,10 +146,28 @@ def _rays(rng, n):
     return x
 
 
-def test_attempts_bit_identical(dev):
+def test_sums(dev):
+    """s + f for floats of every size below and around the line to native
+    sums, and r - 2 around 1, 2, 4, 2^52 and the ends of its range."""
+    rng = np.random.default_rng(17)
+    s = np.concatenate([_numbers(rng, 60000, 60), _numbers(rng, 30000, 60, 4),
+                        2.0 ** rng.integers(-2, 56, 30000) *
+                        (1.0 + rng.integers(-3, 4, 30000) * 2.0 ** -52)])
+    ratio = 2.0 ** -rng.integers(0, 75, s.size).astype(np.float64)
+    f = (s * ratio * rng.uniform(0.5, 2.0, s.size) * rng.choice([-1.0, 1.0], s.size))
+    f = f.astype(np.float32)
+    f[::11] = 0.0
+    f[1::11] = np.ldexp(1.0, np.frexp(f[1::11])[1]).astype(np.float32)  # powers of two
+    got = dev("a", np.stack([s, f.astype(np.float64)], 1), 2)
+    want = np.stack([s + f.astype(np.float64), np.abs(s) - 2.0], 1)
+    assert np.array_equal(got.copy().view(np.uint64), want.view(np.uint64))
+
+
+@pytest.mark.parametrize("sums", ["s", "n"])
+def test_attempts_bit_identical(dev, sums):
     rng = np.random.default_rng(11)
     x = _rays(rng, 16000)
-    out = dev("s", x, 23)
+    out = dev(sums, x, 23)
     kept = out[:, 22] == 0
     # a random step next to the horizon may throw a stage far out: 1 of these 16,000
     assert (~kept).sum() <= 4
