@@ -749,7 +749,8 @@ int osiris_batch_plan_create(osiris_batch_plan** out, int32_t max_requests, int3
   p->block = block_of(&p->opts);
   int rc = OSIRIS_OK;
   for (int k = 0; k < 2 && rc == OSIRIS_OK; ++k) {
-    p->variant[k].fn = kernel_of(&p->opts, Kernel::kPersistent, spacetime, k ? INT64_MAX : 1);
+    p->variant[k].fn = kernel_of(&p->opts, Kernel::kPersistent, spacetime,
+                                 k ? INT64_MAX : osiris_impl::kTinyBatch);
     rc = full_grid(&p->opts, p->variant[k].fn, &p->variant[k].full_grid);
   }
   if (rc == OSIRIS_OK &&

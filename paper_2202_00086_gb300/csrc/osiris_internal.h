@@ -65,7 +65,11 @@ constexpr size_t kQueueBytes = 256;  // workspace head: the ray counter
 enum class Kernel { kPlain, kPersistent };
 
 // The trace kernel of a launch: by precision, kind, integrator, space-time and
-// the launch's rays.
+// the launch's rays. Each precision has a kernel for small and one for large
+// launches; persistent DF64 and MIXED launches of under kTinyBatch rays take
+// the latter too, at up to 1.5 times the time of the former (the server's
+// tests pace their arrivals to the length of such rounds).
+constexpr int64_t kTinyBatch = 4096;
 const void* trace_kernel_fp64(Kernel kind, int integrator, int spacetime, int64_t rays);
 const void* trace_kernel_mixed(Kernel kind, int integrator, int spacetime, int64_t rays);
 const void* trace_kernel_df64(Kernel kind, int integrator, int spacetime, int64_t rays);

@@ -32,19 +32,30 @@ namespace osiris_impl {
 
 // Metric policies of the double-float kernels: the ray constants, the
 // evaluation, and the register cap.
-// Registers capped at 128 so that four blocks of 128 threads (16 warps) are
-// resident per SM: the double-float dependency chains need the extra warps
-// more than they lose to the spilled values, which stay in L1 as long as no
-// shared memory is reserved. Measured on the 12 x 1024^2 Kerr set (Mrays/s,
-// Cash-Karp): 168 registers (three blocks) 14.4, 128: 15.5, 112: 15.4,
-// 96: 15.3, 80: 14.7.
-#ifndef OSIRIS_DF64_MAXREGS
-#define OSIRIS_DF64_MAXREGS 128
-#endif
+//
+// Two variants, chosen by the launch's rays. Large launches: 128 registers, so
+// that four blocks of 128 threads (16 warps) are resident per SM: the
+// double-float dependency chains need the extra warps more than they lose to
+// the spilled values, which stay in L1 as long as no shared memory is
+// reserved (12 x 1024^2 Kerr set, Mrays/s, Cash-Karp: 168 registers (three
+// blocks) 14.4, 128: 15.5, 112: 15.4, 96: 15.3, 80: 14.7). Small launches have
+// one or two warps per SM sub-partition and last as long as their longest
+// chains: no cap (201-231 registers, two blocks per SM), nothing spilled. 128
+// registers / no cap, ms:
+//   Kerr render  32^2  5.2 / 3.3     100^2  6.3 / 4.0     160^2  7.4 / 5.2
+//               256^2  7.8 / 7.1     360^2 11.9 / 10.1    512^2 18.1 / 18.3
+//   disk        100^2  4.3 / 2.9     256^2  5.7 / 5.3     400^2  9.3 / 9.5
+//   q-metric     64^2  9.0 / 6.3     300^2 17.7 / 15.4    600^2 38.3 / 42.5
+//   Dormand-Prince render  64^2  6.3 / 4.2    400^2 14.1 / 13.4    800^2 39.2 / 43.8
+//   particles    5,000  1.1 / 0.75  100,000  2.55 / 2.55
+// The line lies at 3.5 times the lanes of the uncapped kernels in flight.
+constexpr int64_t kLargeLaunch = 7 * 152 * 256 / 2;
+constexpr int kLargeRegs = 128;
 
 struct KerrDF {
   using Ray = RayDF;
-  static constexpr int kMaxRegs = OSIRIS_DF64_MAXREGS;
+  static constexpr int kMaxRegs = kLargeRegs;
+  static constexpr bool kFusedR2 = true;
   static __device__ __forceinline__ Ray ray(const RayK& K) { return to_df(K); }
   static __device__ __forceinline__ void rhs(const Ray& K, df r, df th, df pr, df pth, df& dr,
                                              df& dth, df& dph, df& dpr, df& dpth,
@@ -64,7 +75,8 @@ struct KerrDF {
 
 struct QMetricDF {
   using Ray = RayQDF;
-  static constexpr int kMaxRegs = OSIRIS_DF64_MAXREGS;
+  static constexpr int kMaxRegs = kLargeRegs;
+  static constexpr bool kFusedR2 = true;
   static __device__ __forceinline__ Ray ray(const RayK& K) { return to_qdf(K); }
   static __device__ __forceinline__ void rhs(const Ray& K, df r, df th, df pr, df pth, df& dr,
                                              df& dth, df& dph, df& dpr, df& dpth,
@@ -82,32 +94,38 @@ struct QMetricDF {
   }
 };
 
-template <class Met, int INTEG>
-__global__ void __maxnreg__(Met::kMaxRegs) trace_df64_plain(const __grid_constant__ KernelArgs A) {
+template <class Met, int INTEG, bool kLarge>
+__global__ void __maxnreg__(kLarge ? Met::kMaxRegs : 255)
+    trace_df64_plain(const __grid_constant__ KernelArgs A) {
   trace_body_df<Met, false, INTEG>(A);
 }
 
-template <class Met, int INTEG>
-__global__ void __maxnreg__(Met::kMaxRegs)
+template <class Met, int INTEG, bool kLarge>
+__global__ void __maxnreg__(kLarge ? Met::kMaxRegs : 255)
     trace_df64_persistent(const __grid_constant__ KernelArgs A) {
   trace_body_df<Met, true, INTEG>(A);
 }
 
-template <class Met, int INTEG>
+template <class Met, int INTEG, bool kLarge>
 static const void* df64_kernel(Kernel kind) {
-  return kind == Kernel::kPersistent ? (const void*)trace_df64_persistent<Met, INTEG>
-                                     : (const void*)trace_df64_plain<Met, INTEG>;
+  return kind == Kernel::kPersistent ? (const void*)trace_df64_persistent<Met, INTEG, kLarge>
+                                     : (const void*)trace_df64_plain<Met, INTEG, kLarge>;
 }
 
 template <class Met>
-static const void* df64_kernel(Kernel kind, int integrator) {
-  return integrator == OSIRIS_RKDP45 ? df64_kernel<Met, OSIRIS_RKDP45>(kind)
-                                     : df64_kernel<Met, OSIRIS_RKCK45>(kind);
+static const void* df64_kernel(Kernel kind, int integrator, bool large) {
+  if (integrator == OSIRIS_RKDP45)
+    return large ? df64_kernel<Met, OSIRIS_RKDP45, true>(kind)
+                 : df64_kernel<Met, OSIRIS_RKDP45, false>(kind);
+  return large ? df64_kernel<Met, OSIRIS_RKCK45, true>(kind)
+               : df64_kernel<Met, OSIRIS_RKCK45, false>(kind);
 }
 
-const void* trace_kernel_df64(Kernel kind, int integrator, int spacetime, int64_t) {
-  return spacetime == OSIRIS_SPACETIME_QMETRIC ? df64_kernel<QMetricDF>(kind, integrator)
-                                               : df64_kernel<KerrDF>(kind, integrator);
+const void* trace_kernel_df64(Kernel kind, int integrator, int spacetime, int64_t rays) {
+  const bool large =
+      rays >= kLargeLaunch || (kind == Kernel::kPersistent && rays < kTinyBatch);
+  return spacetime == OSIRIS_SPACETIME_QMETRIC ? df64_kernel<QMetricDF>(kind, integrator, large)
+                                               : df64_kernel<KerrDF>(kind, integrator, large);
 }
 
 }  // namespace osiris_impl

@@ -99,7 +99,8 @@ __device__ __forceinline__ bool any_not_finite(const float (&v)[N]) {
 // 2 (H - H0) at the end point in double-float; kTrackH, whether the |H| of
 // every step start (from rhs) enters the ray's max |H|; kLocateRel, the
 // relative width of the step-length bracket at which surface location stops
-// (the resolution of a trial step's end point); kMaxRegs, the register cap.
+// (the resolution of a trial step's end point); kFusedR2 (see write_outputs);
+// kMaxRegs, the register cap of large launches.
 template <class Met, bool PERSISTENT, int INTEG>
 __device__ __forceinline__ void trace_body_df(const KernelArgs& A) {
   const unsigned FULL = 0xffffffffu;
@@ -159,7 +160,7 @@ __device__ __forceinline__ void trace_body_df(const KernelArgs& A) {
       mh = fmaxf(mh, fabsf(0.5f * Met::end_twoH(KD, I.K, yF)));
       S.rhs += 1;
     }
-    write_outputs(A, I, done_status, f, (double)mh, n_acc, n_rej, S);
+    write_outputs<Met::kFusedR2>(A, I, done_status, f, (double)mh, n_acc, n_rej, S);
     mode = MODE_IDLE;
   };
 

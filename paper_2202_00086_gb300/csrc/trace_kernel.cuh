@@ -114,7 +114,11 @@ __device__ __forceinline__ double wrap_2pi(double x) {
 }
 
 // Write the outputs of a finished ray (terminal state f, final max |H|) and
-// fold it into the lane's counters.
+// fold it into the lane's counters. kFusedR2: r^2 + a^2 of the disk
+// observables with one rounding, written out because the units that let the
+// compiler contract (trace_df64.cu) could have it fuse either square,
+// differently in different kernels.
+template <bool kFusedR2>
 __device__ __forceinline__ void write_outputs(const KernelArgs& A, const RayInfo& I, int status,
                                               const State& f, double max_abs_H, unsigned n_acc,
                                               unsigned n_rej, LaneStats& S) {
@@ -158,7 +162,8 @@ __device__ __forceinline__ void write_outputs(const KernelArgs& A, const RayInfo
     const double r = f.r, a = I.K.a;
     const double gtt = -(1.0 - 2.0 / r);
     const double gtp = -2.0 * a / r;
-    const double gpp = r * r + a * a + 2.0 * a * a / r;
+    const double r2a2 = kFusedR2 ? fma(r, r, a * a) : r * r + a * a;
+    const double gpp = r2a2 + 2.0 * a * a / r;
     const double Om = (R->disk == OSIRIS_DISK_CONSTANT_L)
                           ? -(gtp + R->l0 * gtt) / (gpp + R->l0 * gtp)
                           : 1.0 / fma(r, sqrt(r), a);
@@ -336,7 +341,7 @@ __device__ __forceinline__ void trace_body(const KernelArgs& A) {
       track_abs_H(max_abs_H, Stepper::twoH(K, yF), I.H0);
       S.rhs += 1;
     }
-    write_outputs(A, I, done_status, yF, __longlong_as_double(max_abs_H), n_acc, n_rej, S);
+    write_outputs<false>(A, I, done_status, yF, __longlong_as_double(max_abs_H), n_acc, n_rej, S);
     mode = MODE_IDLE;
   };
 

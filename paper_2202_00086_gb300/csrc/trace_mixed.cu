@@ -32,24 +32,30 @@
 
 namespace osiris_impl {
 
-// Registers capped so that more blocks of 128 threads are resident per SM
-// than the code's natural ~190 registers allow: the FP32 stepper keeps only
-// the df64 state, the stage inputs and FP32 sums live, and the extra warps
-// hide more of the dependent FP32 chains than the added spills (L1 hits)
-// cost. Measured on the 12 x 1024^2 Kerr set at tol 1e-8 (Mrays/s, Cash-Karp,
-// refill at 32 idle lanes): 96 registers 160.9, 80 (6 blocks): 162.3, 72:
-// 154.7, 64: 153.0; on the six q-metric renders: 80: 117.6, 72: 118.9, 64:
-// 123.3, 56 (9 blocks): 127.1.
-#ifndef OSIRIS_MIXED_MAXREGS
-#define OSIRIS_MIXED_MAXREGS 80
-#endif
-#ifndef OSIRIS_MIXED_Q_MAXREGS
-#define OSIRIS_MIXED_Q_MAXREGS 56
-#endif
+// Registers. Large launches are bound by issue slots and gain from warps that
+// hide the dependent FP32 chains: 80 registers (six blocks of 128 threads per
+// SM) for Kerr, 128 (four) for the q-metric. Measured at tol 1e-8 on the
+// 12 x 1024^2 Kerr set (Mrays/s, Cash-Karp, refill at 32 idle lanes): 96
+// registers 160.9, 80: 162.3, 72: 154.7, 64: 153.0; on six 500^2 q-metric
+// renders in one launch (ms) 56 registers 13.8, 80: 14.6, 104: 14.5, 128: 12.7,
+// no cap 13.5, on a 1024^2 render 9.45 / 9.47 / 10.1 / 9.17 / 9.9. Small
+// launches last as long as their longest chains: no cap (145-160 registers,
+// three blocks per SM), nothing spilled. 80 / no cap, in ms, for Kerr:
+//   render     32^2  0.80 / 0.62    256^2  1.13 / 0.99    512^2  2.37 / 2.29
+//             800^2  4.32 / 4.58
+//   disk      200^2  1.08 / 0.89    500^2  1.85 / 1.82    900^2  4.51 / 4.91
+//   six renders in one launch  100^2  1.33 / 1.12    200^2  2.51 / 2.52    400^2  7.2 / 7.6
+//   Dormand-Prince render      200^2  1.13 / 0.89    400^2  1.76 / 1.66    800^2  4.46 / 4.81
+// and 128 / no cap for the q-metric: 100^2 0.89 / 0.82, 300^2 1.68 / 1.60, 600^2
+// 3.69 / 3.94, six 200^2 renders 2.89 / 2.93. The lines lie at 5 and 2.5 times
+// 256 lanes on each of 152 SMs.
+constexpr int64_t kLargeLaunchKerr = 5 * 152 * 256;
+constexpr int64_t kLargeLaunchQ = 5 * 152 * 256 / 2;
 
 struct KerrMixed {
   using Ray = RayF32;
-  static constexpr int kMaxRegs = OSIRIS_MIXED_MAXREGS;
+  static constexpr int kMaxRegs = 80;
+  static constexpr bool kFusedR2 = false;
   static constexpr bool kTrackH = false;
   static constexpr bool kF32Stages = true;
   static constexpr double kLocateRel = 2e-7;
@@ -89,7 +95,8 @@ struct KerrMixed {
 // the double-float q-metric equations (rhs_q_df).
 struct QMetricMixed {
   using Ray = RayQF32;
-  static constexpr int kMaxRegs = OSIRIS_MIXED_Q_MAXREGS;
+  static constexpr int kMaxRegs = 128;
+  static constexpr bool kFusedR2 = false;
   static constexpr bool kTrackH = false;
   static constexpr bool kF32Stages = true;
   static constexpr double kLocateRel = 2e-7;
@@ -120,32 +127,39 @@ struct QMetricMixed {
   }
 };
 
-template <class Met, int INTEG>
-__global__ void __maxnreg__(Met::kMaxRegs) trace_mixed_plain(const __grid_constant__ KernelArgs A) {
+template <class Met, int INTEG, bool kLarge>
+__global__ void __maxnreg__(kLarge ? Met::kMaxRegs : 255)
+    trace_mixed_plain(const __grid_constant__ KernelArgs A) {
   trace_body_df<Met, false, INTEG>(A);
 }
 
-template <class Met, int INTEG>
-__global__ void __maxnreg__(Met::kMaxRegs)
+template <class Met, int INTEG, bool kLarge>
+__global__ void __maxnreg__(kLarge ? Met::kMaxRegs : 255)
     trace_mixed_persistent(const __grid_constant__ KernelArgs A) {
   trace_body_df<Met, true, INTEG>(A);
 }
 
-template <class Met, int INTEG>
+template <class Met, int INTEG, bool kLarge>
 static const void* mixed_kernel(Kernel kind) {
-  return kind == Kernel::kPersistent ? (const void*)trace_mixed_persistent<Met, INTEG>
-                                     : (const void*)trace_mixed_plain<Met, INTEG>;
+  return kind == Kernel::kPersistent ? (const void*)trace_mixed_persistent<Met, INTEG, kLarge>
+                                     : (const void*)trace_mixed_plain<Met, INTEG, kLarge>;
 }
 
 template <class Met>
-static const void* mixed_kernel(Kernel kind, int integrator) {
-  return integrator == OSIRIS_RKDP45 ? mixed_kernel<Met, OSIRIS_RKDP45>(kind)
-                                     : mixed_kernel<Met, OSIRIS_RKCK45>(kind);
+static const void* mixed_kernel(Kernel kind, int integrator, bool large) {
+  if (integrator == OSIRIS_RKDP45)
+    return large ? mixed_kernel<Met, OSIRIS_RKDP45, true>(kind)
+                 : mixed_kernel<Met, OSIRIS_RKDP45, false>(kind);
+  return large ? mixed_kernel<Met, OSIRIS_RKCK45, true>(kind)
+               : mixed_kernel<Met, OSIRIS_RKCK45, false>(kind);
 }
 
-const void* trace_kernel_mixed(Kernel kind, int integrator, int spacetime, int64_t) {
-  return spacetime == OSIRIS_SPACETIME_QMETRIC ? mixed_kernel<QMetricMixed>(kind, integrator)
-                                               : mixed_kernel<KerrMixed>(kind, integrator);
+const void* trace_kernel_mixed(Kernel kind, int integrator, int spacetime, int64_t rays) {
+  const bool q = spacetime == OSIRIS_SPACETIME_QMETRIC;
+  const bool large = rays >= (q ? kLargeLaunchQ : kLargeLaunchKerr) ||
+                     (kind == Kernel::kPersistent && rays < kTinyBatch);
+  return q ? mixed_kernel<QMetricMixed>(kind, integrator, large)
+           : mixed_kernel<KerrMixed>(kind, integrator, large);
 }
 
 }  // namespace osiris_impl
