@@ -145,6 +145,8 @@ __device__ __forceinline__ double exact_of(long long x, int k) {
 // Plain FP64 instructions: the end point of a ray, and the attempts that
 // ArithFast gives back.
 struct ArithPlain {
+  static constexpr bool kRolledSums = false;
+  static constexpr double nz = -0.0;
   __device__ __forceinline__ double mul(double a, double b) const { return a * b; }
   __device__ __forceinline__ double soft(double a, double b) const { return a * b; }
   __device__ __forceinline__ double soft0(double a, double b) const { return a * b; }
@@ -174,6 +176,7 @@ static inline double rare_add(double a, double c) { return a + c; }
 // hide that (kLargeLaunch in trace_fp64.cu).
 template <bool kSums>
 struct ArithFast {
+  static constexpr bool kRolledSums = kSums;  // see rk_attempt64
   double one, nz;
   unsigned range;  // collects the exponent bits that leave the window
 

@@ -534,6 +534,11 @@ OSIRIS_TABLEAU64 double kDormandPrinceA[6][6] = {
     {dp::A41, dp::A42, dp::A43, 0, 0, 0},
     {dp::A51, dp::A52, dp::A53, dp::A54, 0, 0},
     {dp::A61, dp::A62, dp::A63, dp::A64, dp::A65, 0}};  // the seventh stage is evaluated at o
+// The weights b (fifth order) and e (fifth minus embedded fourth order) of both.
+OSIRIS_TABLEAU64 double kWeights64[2][2][7] = {
+    {{ck::B1, 0, ck::B3, ck::B4, 0, ck::B6, 0}, {ck::D1, 0, ck::D3, ck::D4, ck::D5, ck::D6, 0}},
+    {{dp::B1, 0, dp::B3, dp::B4, dp::B5, dp::B6, 0},
+     {dp::D1, 0, dp::D3, dp::D4, dp::D5, dp::D6, dp::D7}}};
 #undef OSIRIS_TABLEAU64
 
 struct CashKarp64 {
@@ -573,7 +578,9 @@ struct DormandPrince64 {
 // the integer pipes do not fit (the q-metric's least of all). Measured with
 // plain FP64 multiplies and six copies / products on the integer pipes and
 // six copies / and one copy: twelve 320^2 Kerr renders in one launch 338 /
-// 267 / 248 ms, a 333 x 257 q-metric render 57.3 / 59.9 / 44.2 ms.
+// 267 / 248 ms, a 333 x 257 q-metric render 57.3 / 59.9 / 44.2 ms. The large
+// variant (A::kRolledSums) rolls the sums of the result and of the error, too:
+// twelve 640^2 renders 857 -> 831 ms; the small one is 4 % slower that way.
 template <class Met, class Tab, class A>
 __device__ __forceinline__ void rk_attempt64(const RayK& K, const State& y, double h,
                                              bool have_first, Deriv& first, State& o, State& d,
@@ -591,18 +598,35 @@ __device__ __forceinline__ void rk_attempt64(const RayK& K, const State& y, doub
     k[0] = {first.r, first.th, first.ph, first.pr, first.pth,
             Met::kUnitScale ? h : ar.soft(h, first.scale)};
   }
+  // o += b_j w_j k~_j and d += e_j w_j k~_j; a product is the sum with -0
+  auto add_result = [&](double b, int j) {
+    const double c = ar.soft(b, k[j].w);
+    o.r = fma(c, k[j].r, o.r);
+    o.th = fma(c, k[j].th, o.th);
+    o.ph = fma(c, k[j].ph, o.ph);
+    o.pr = fma(c, k[j].pr, o.pr);
+    o.pth = fma(c, k[j].pth, o.pth);
+  };
+  auto add_error = [&](double e, int j) {
+    const double c = ar.soft(e, k[j].w);
+    d.r = fma(c, k[j].r, d.r);
+    d.th = fma(c, k[j].th, d.th);
+    d.ph = fma(c, k[j].ph, d.ph);
+    d.pr = fma(c, k[j].pr, d.pr);
+    d.pth = fma(c, k[j].pth, d.pth);
+  };
   auto fifth_order = [&]() {
     o = y;
-#pragma unroll
-    for (int j = 0; j < NI; ++j) {
-      if (Tab::b(j) != 0.0) {
-        const double c = ar.soft(Tab::b(j), k[j].w);
-        o.r = fma(c, k[j].r, o.r);
-        o.th = fma(c, k[j].th, o.th);
-        o.ph = fma(c, k[j].ph, o.ph);
-        o.pr = fma(c, k[j].pr, o.pr);
-        o.pth = fma(c, k[j].pth, o.pth);
+    if (A::kRolledSums) {
+#pragma unroll 1
+      for (int j = 0; j < NI; ++j) {
+        const double b = kWeights64[Tab::kFsal][0][j];
+        if (bits_of(b) != 0) add_result(b, j);
       }
+    } else {
+#pragma unroll
+      for (int j = 0; j < NI; ++j)
+        if (Tab::b(j) != 0.0) add_result(Tab::b(j), j);
     }
   };
 #pragma unroll 1
@@ -631,22 +655,17 @@ __device__ __forceinline__ void rk_attempt64(const RayK& K, const State& y, doub
     if (s == NS - 1) last = ks;
   }
   if (!Tab::kFsal) fifth_order();
-  const double c0 = ar.soft(Tab::e(0), k[0].w);
-  d.r = ar.mul(c0, k[0].r);
-  d.th = ar.mul(c0, k[0].th);
-  d.ph = ar.mul(c0, k[0].ph);
-  d.pr = ar.mul(c0, k[0].pr);
-  d.pth = ar.mul(c0, k[0].pth);
-#pragma unroll
-  for (int j = 1; j < NS; ++j) {
-    if (Tab::e(j) != 0.0) {
-      const double c = ar.soft(Tab::e(j), k[j].w);
-      d.r = fma(c, k[j].r, d.r);
-      d.th = fma(c, k[j].th, d.th);
-      d.ph = fma(c, k[j].ph, d.ph);
-      d.pr = fma(c, k[j].pr, d.pr);
-      d.pth = fma(c, k[j].pth, d.pth);
+  d.r = d.th = d.ph = d.pr = d.pth = ar.nz;
+  if (A::kRolledSums) {
+#pragma unroll 1
+    for (int j = 0; j < NS; ++j) {
+      const double e = kWeights64[Tab::kFsal][1][j];
+      if (bits_of(e) != 0) add_error(e, j);
     }
+  } else {
+#pragma unroll
+    for (int j = 0; j < NS; ++j)
+      if (Tab::e(j) != 0.0) add_error(Tab::e(j), j);
   }
 }
 
