@@ -187,6 +187,19 @@ int full_grid(const osiris_trace_opts* o, const void* fn, int64_t* grid) {
 constexpr int kDefaultRaysPerLane = 1;
 constexpr int kDefaultRefillLanes = 4;
 constexpr int kDefaultRefillLanesMixed = 32;
+// Plain launches that steal: a warp takes 32 rays at a time. Neighbouring
+// pixels take similar numbers of steps, so a warp's lanes start together (32;
+// 4: 400^2 FP64 39.9 against 39.5 ms, 800^2 114 against 109, 640 x 320
+// Dormand-Prince disk 50.7 against 47.8); explicit initial data come in any
+// order, and idle lanes refill four at a time (600,000 particles FP64 29.0
+// against 34.1 ms, DF64 9.2 against 11.0).
+// An index stands for 32 rays, or for a block's (one ray a thread) in launches
+// of up to 1.5 times the lanes of two blocks per SM: most of those blocks are
+// resident at once, and a block's warps lie on different sub-partitions (40,000
+// DF64 rays 5.0 against 5.2 ms).
+constexpr int64_t kStealChunk = 32;
+constexpr int64_t kStealFrom = 3 * 152 * 128;
+constexpr int kRefillLanesStates = 4;
 
 void set_granularity(KernelArgs& args, const osiris_trace_opts* o) {
   args.rays_per_lane = o->rays_per_lane > 0 ? o->rays_per_lane : kDefaultRaysPerLane;
@@ -208,7 +221,17 @@ int launch(KernelArgs& args, const osiris_trace_opts* o, void* stream) {
   if (!persistent) {
     if (needed > 0x7fffffff) return OSIRIS_EINVAL;
     args.queue = nullptr;
-    return launch_kernel(kernel_of(o, Kernel::kPlain, spacetime, args.total_rays), args, needed,
+    int64_t grid = needed;
+    if (o->precision != OSIRIS_MIXED) {  // plain FP64 and DF64 kernels steal (work_steal.cuh)
+      const int64_t small_chunk = kStealChunk * args.rays_per_lane;
+      args.chunk = args.total_rays > kStealFrom &&
+                           args.total_rays <= small_chunk * int64_t{0x7fffffff}
+                       ? small_chunk
+                       : per_block;
+      args.refill_lanes = args.single.explicit_states ? kRefillLanesStates : 32;
+      grid = (args.total_rays + args.chunk - 1) / args.chunk;
+    }
+    return launch_kernel(kernel_of(o, Kernel::kPlain, spacetime, args.total_rays), args, grid,
                          block, s);
   }
   if (!o->workspace || o->workspace_bytes < osiris_impl::kQueueBytes) return OSIRIS_ENOMEM;

@@ -55,14 +55,18 @@ struct KernelArgs {
   unsigned long long* queue;       // persistent grids: next ray index (device)
   unsigned long long* stats;       // optional OSIRIS_STATS_LEN counters (device)
   int32_t rays_per_lane;           // rays a lane claims at once (plain: per thread), >= 1
-  int32_t refill_lanes;            // persistent: idle lanes a warp waits for before it
-                                   // refills (unless none of its lanes is busy), 1..32
+  int32_t refill_lanes;            // persistent, stealing: idle lanes a warp waits for before
+                                   // it refills (unless none of its lanes is busy), 1..32
+  int64_t chunk;                   // stealing: rays that a block index stands for
   ReqDev single;
 };
 
 constexpr size_t kQueueBytes = 256;  // workspace head: the ray counter
 
-enum class Kernel { kPlain, kPersistent };
+// How a launch deals out its rays: one (or rays_per_lane) per thread, a ray
+// queue in memory, or block indices taken from blocks that have not started
+// (work_steal.cuh; the plain FP64 and DF64 launches).
+enum class Kernel { kPlain, kPersistent, kSteal };
 
 // The trace kernel of a launch: by precision, kind, integrator, space-time and
 // the launch's rays. Each precision has a kernel for small and one for large

@@ -97,13 +97,13 @@ struct QMetricDF {
 template <class Met, int INTEG, bool kLarge>
 __global__ void __maxnreg__(kLarge ? Met::kMaxRegs : 255)
     trace_df64_plain(const __grid_constant__ KernelArgs A) {
-  trace_body_df<Met, false, INTEG>(A);
+  trace_body_df<Met, Kernel::kSteal, INTEG>(A);
 }
 
 template <class Met, int INTEG, bool kLarge>
 __global__ void __maxnreg__(kLarge ? Met::kMaxRegs : 255)
     trace_df64_persistent(const __grid_constant__ KernelArgs A) {
-  trace_body_df<Met, true, INTEG>(A);
+  trace_body_df<Met, Kernel::kPersistent, INTEG>(A);
 }
 
 template <class Met, int INTEG, bool kLarge>

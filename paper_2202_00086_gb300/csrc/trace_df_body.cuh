@@ -101,11 +101,12 @@ __device__ __forceinline__ bool any_not_finite(const float (&v)[N]) {
 // relative width of the step-length bracket at which surface location stops
 // (the resolution of a trial step's end point); kFusedR2 (see write_outputs);
 // kMaxRegs, the register cap of large launches.
-template <class Met, bool PERSISTENT, int INTEG>
+template <class Met, Kernel KIND, int INTEG>
 __device__ __forceinline__ void trace_body_df(const KernelArgs& A) {
   const unsigned FULL = 0xffffffffu;
   int mode = MODE_IDLE;
-  bool drained = !PERSISTENT;
+  bool drained = KIND == Kernel::kPlain;
+  unsigned turns_without = 0;  // stealing: turns in a row without any ray
   LaneStats S;
 
   RayInfo I;
@@ -215,16 +216,27 @@ __device__ __forceinline__ void trace_body_df(const KernelArgs& A) {
     }
   };
 
-  init_claim<PERSISTENT>(A);
+  init_claim<KIND>(A);
 
   for (;;) {
     if (complete_finished(A, mode)) complete();
     const bool busy = (mode == MODE_INTEGRATE) || (mode == MODE_LOCATE);
-    if (mode == MODE_IDLE) {
+    if (KIND != Kernel::kSteal && mode == MODE_IDLE) {
       const int64_t g = next_claimed(A);
       if (g >= 0) start_ray(g);
     }
-    if (PERSISTENT) {
+    if (KIND == Kernel::kSteal) {
+      int64_t first = 0;
+      bool over = false;
+      if (steal_refill(A, (mode == MODE_IDLE) && !drained, busy, first, over)) start_ray(first);
+      drained |= over;
+      if (!__any_sync(FULL, mode != MODE_IDLE)) {
+        if (drained || ++turns_without > kStealPatience) break;
+        continue;
+      }
+      turns_without = 0;
+    }
+    if (KIND == Kernel::kPersistent) {
       int64_t first = 0;
       const int got = refill(A, (mode == MODE_IDLE) && !drained, busy, first);
       if (got > 0) {
@@ -234,7 +246,7 @@ __device__ __forceinline__ void trace_body_df(const KernelArgs& A) {
         drained = true;
       }
     }
-    if (!__any_sync(FULL, mode != MODE_IDLE || has_claim())) break;
+    if (KIND != Kernel::kSteal && !__any_sync(FULL, mode != MODE_IDLE || has_claim())) break;
     if (mode != MODE_INTEGRATE && mode != MODE_LOCATE) continue;
 
     const float hs_f = fminf(h, 0.1f * y.r.hi);

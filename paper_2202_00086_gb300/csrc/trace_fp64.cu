@@ -135,13 +135,13 @@ constexpr int64_t kLargeLaunch = 5 * 152 * 256;
 template <int INTEG, class Met, bool kLarge>
 __global__ void __maxnreg__(kLarge ? 128 : 255)
     trace_fp64_plain(const __grid_constant__ KernelArgs A) {
-  trace_body<StepperFP64<INTEG, Met, kLarge>, false>(A);
+  trace_body<StepperFP64<INTEG, Met, kLarge>, Kernel::kSteal>(A);
 }
 
 template <int INTEG, class Met, bool kLarge>
 __global__ void __maxnreg__(kLarge ? 128 : 255)
     trace_fp64_persistent(const __grid_constant__ KernelArgs A) {
-  trace_body<StepperFP64<INTEG, Met, kLarge>, true>(A);
+  trace_body<StepperFP64<INTEG, Met, kLarge>, Kernel::kPersistent>(A);
 }
 
 template <int INTEG, class Met, bool kLarge>

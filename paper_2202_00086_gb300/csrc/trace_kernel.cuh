@@ -14,6 +14,7 @@
 
 #include "checked.cuh"
 #include "trace_device.cuh"
+#include "work_steal.cuh"
 
 namespace osiris_impl {
 
@@ -244,8 +245,10 @@ __device__ __forceinline__ LaneClaims& lane_claims() {
 // The lane's first claim: a plain launch (one launch thread per ray range)
 // gives each thread rays_per_lane consecutive rays from thread index x
 // rays_per_lane; a persistent grid starts with none and refills.
-template <bool PERSISTENT>
+template <Kernel KIND>
 __device__ __forceinline__ void init_claim(const KernelArgs& A) {
+  if (KIND == Kernel::kSteal) return steal_init(A);
+  constexpr bool PERSISTENT = KIND == Kernel::kPersistent;
   LaneClaims& C = lane_claims();
   long long next = 0, end = 0;
   if (!PERSISTENT) {
@@ -279,7 +282,7 @@ __device__ __forceinline__ void set_claim(int64_t first, int count) {
   C.end[threadIdx.x] = first + count;
 }
 
-template <class Stepper, bool PERSISTENT>
+template <class Stepper, Kernel KIND>
 __device__ __forceinline__ void trace_body(const KernelArgs& A) {
   const unsigned FULL = 0xffffffffu;
   if (Stepper::kTrigTable) trig_table_init();
@@ -288,7 +291,8 @@ __device__ __forceinline__ void trace_body(const KernelArgs& A) {
   const double one = fma_units().one, nz = fma_units().nz;
 
   int mode = MODE_IDLE;
-  bool drained = !PERSISTENT;
+  bool drained = KIND == Kernel::kPlain;
+  unsigned turns_without = 0;  // stealing: turns in a row without any ray
   LaneStats S;
 
   // ray identity and constants
@@ -379,16 +383,27 @@ __device__ __forceinline__ void trace_body(const KernelArgs& A) {
     }
   };
 
-  init_claim<PERSISTENT>(A);
+  init_claim<KIND>(A);
 
   for (;;) {
     if (complete_finished(A, mode)) complete();
     const bool busy = (mode == MODE_INTEGRATE) || (mode == MODE_LOCATE);
-    if (mode == MODE_IDLE) {
+    if (KIND != Kernel::kSteal && mode == MODE_IDLE) {
       const int64_t g = next_claimed(A);
       if (g >= 0) start_ray(g);
     }
-    if (PERSISTENT) {
+    if (KIND == Kernel::kSteal) {
+      int64_t first = 0;
+      bool over = false;
+      if (steal_refill(A, (mode == MODE_IDLE) && !drained, busy, first, over)) start_ray(first);
+      drained |= over;
+      if (!__any_sync(FULL, mode != MODE_IDLE)) {
+        if (drained || ++turns_without > kStealPatience) break;
+        continue;
+      }
+      turns_without = 0;
+    }
+    if (KIND == Kernel::kPersistent) {
       int64_t first = 0;
       const int got = refill(A, (mode == MODE_IDLE) && !drained, busy, first);
       if (got > 0) {
@@ -398,7 +413,7 @@ __device__ __forceinline__ void trace_body(const KernelArgs& A) {
         drained = true;
       }
     }
-    if (!__any_sync(FULL, mode != MODE_IDLE || has_claim())) break;
+    if (KIND != Kernel::kSteal && !__any_sync(FULL, mode != MODE_IDLE || has_claim())) break;
     if (mode != MODE_INTEGRATE && mode != MODE_LOCATE) continue;
 
     // (a ray with a non-finite r ends at this attempt whatever its length)

@@ -130,13 +130,13 @@ struct QMetricMixed {
 template <class Met, int INTEG, bool kLarge>
 __global__ void __maxnreg__(kLarge ? Met::kMaxRegs : 255)
     trace_mixed_plain(const __grid_constant__ KernelArgs A) {
-  trace_body_df<Met, false, INTEG>(A);
+  trace_body_df<Met, Kernel::kPlain, INTEG>(A);
 }
 
 template <class Met, int INTEG, bool kLarge>
 __global__ void __maxnreg__(kLarge ? Met::kMaxRegs : 255)
     trace_mixed_persistent(const __grid_constant__ KernelArgs A) {
-  trace_body_df<Met, true, INTEG>(A);
+  trace_body_df<Met, Kernel::kPersistent, INTEG>(A);
 }
 
 template <class Met, int INTEG, bool kLarge>
