@@ -104,10 +104,20 @@ constexpr long long kShiftBits = 0x4338000000000000LL;
 // 1/3 as a float pair, for the log1p series
 constexpr float kThirdH = 0.3333333432674408f, kThirdL = -9.934107758624577e-09f;
 
+// The library's functions, out of line (see rare_sincos in trace_device.cuh).
+#ifdef __CUDACC__
+static __device__ __noinline__ double rare_exp(double y) { return exp(y); }
+static __device__ __noinline__ double rare_log(double x) { return log(x); }
+#else
+static inline double rare_exp(double y) { return exp(y); }
+static inline double rare_log(double x) { return log(x); }
+#endif
+
 template <class A = osiris_impl::ArithPlain>
 __device__ __forceinline__ double exp_tab(double y, const double* t2, A&& ar = A()) {
   using namespace osiris_impl;
-  if (!(fabs(y) < 700.0)) return exp(y);
+  // (comparisons of bits: an FP64 comparison takes the FP64 unit's time)
+  if ((to_bits(y) & 0x7fffffffffffffffLL) >= 0x4085e00000000000LL) return rare_exp(y);  // 700
   const double t = fma(y, kInvL, kShift);
   const int n = (int)(to_bits(t) & 0xffffffffLL);  // y * 64/ln2 rounded, mod 2^32
   const double nd = ar.sub(t, kShift);
@@ -128,8 +138,8 @@ __device__ __forceinline__ double exp_tab(double y, const double* t2, A&& ar = A
 template <class A = osiris_impl::ArithPlain>
 __device__ __forceinline__ double log_tab(double x, const LogEntry* lg, A&& ar = A()) {
   using namespace osiris_impl;
-  if (!(x >= 0x1p-1000 && x <= 0x1p+1000)) return log(x);
   const long long b = to_bits(x);
+  if (b < 0x0170000000000000LL || b > 0x7e70000000000000LL) return rare_log(x);  // 2^+-1000
   const int hi = (int)(b >> 32);
   const double m = from_bits((b & 0x000fffffffffffffLL) | 0x3ff0000000000000LL);
   const int j = ((hi & 0xfffff) + 0x1000) >> 13;  // nearest multiple of 1/128, 0..128

@@ -241,6 +241,21 @@ __device__ __forceinline__ double node_difference(double th, uint64_t n62, int i
   return exact_of((long long)((m << shift) - n62), -62);
 }
 
+// The library's sine and cosine, out of line: inlined, its hundreds of
+// instructions lie in the middle of the attempt loop (with the other library
+// functions and divisions out of line, and the range tests of exp_tab and
+// log_tab on bits: 600^2 q-metric render 167.6 -> 155.5 ms, twelve 640^2 Kerr
+// renders 830 -> 824).
+#ifdef __CUDACC__
+static __device__ __noinline__ double2 rare_sincos(double th) {
+#else
+static inline double2 rare_sincos(double th) {
+#endif
+  double s, c;
+  sincos(th, &s, &c);
+  return make_double2(s, c);
+}
+
 template <class A = ArithPlain>
 __device__ __forceinline__ void sincos_tab(double th, double& s, double& c, A&& ar = A()) {
   using namespace dfc;
@@ -249,7 +264,9 @@ __device__ __forceinline__ void sincos_tab(double th, double& s, double& c, A&& 
                         12582912.0f);
   const int idx = (__float_as_int(tk) - 0x4B400000) - kTrigFirst;
   if ((unsigned)idx >= (unsigned)kTrigNodes) {  // also NaN / inf
-    sincos(th, &s, &c);
+    const double2 sc = rare_sincos(th);
+    s = sc.x;
+    c = sc.y;
     return;
   }
   const TrigTable& t = trig_table();
@@ -277,6 +294,12 @@ __device__ __forceinline__ void track_abs_H(long long& max_bits, double twoH, do
   if (b <= 0x7ff0000000000000LL && b > max_bits) max_bits = b;
 }
 
+#ifdef __CUDACC__
+static __device__ __noinline__ double rare_reciprocal(double d) { return 1.0 / d; }
+#else
+static inline double rare_reciprocal(double d) { return 1.0 / d; }
+#endif
+
 // 1/d: FP32 seed x0 (|x0 d - 1| < 2^-21), then one Newton step with the
 // cubic term, x0 (1 + e + e^2) with e = 1 - d x0, relative error e^3 plus
 // the final rounding (3 FP64 instructions). Outside the FP32 range: 1/d.
@@ -284,7 +307,7 @@ template <class A = ArithPlain>
 __device__ __forceinline__ double rcp64(double d, A&& ar = A()) {
   const long long b = __double_as_longlong(d);
   const int e = (int)((b >> 52) & 0x7ff) - 1023 + 127;
-  if (e < 2 || e > 252) return 1.0 / d;
+  if (e < 2 || e > 252) return rare_reciprocal(d);
   const float f = __int_as_float((int)((b >> 32) & 0x80000000) | (e << 23) |
                                  (int)((b >> 29) & 0x7fffff));
   float rf;
@@ -762,13 +785,17 @@ __device__ __forceinline__ bool less_than_positive(double a, double b) {
   return bits_of(a) < bits_of(b);
 }
 
-// The smaller of two values that are not NaN, on the integer pipe: the bits
-// of a negative double order backwards, so all but its sign are flipped.
+// An integer that orders as the double does (-0 before 0, NaN outside all):
+// the bits of a negative double order backwards, so all but its sign are
+// flipped.
+__device__ __forceinline__ long long ordered(double x) {
+  const long long b = bits_of(x);
+  return b ^ ((b >> 63) & 0x7fffffffffffffffLL);
+}
+
+// The smaller of two values that are not NaN, on the integer pipe.
 __device__ __forceinline__ double min_by_bits(double a, double b) {
-  const long long ia = bits_of(a), ib = bits_of(b);
-  const long long ka = ia ^ ((ia >> 63) & 0x7fffffffffffffffLL);
-  const long long kb = ib ^ ((ib >> 63) & 0x7fffffffffffffffLL);
-  return kb < ka ? b : a;
+  return ordered(b) < ordered(a) ? b : a;
 }
 
 // The sign of cos(theta) changes between two finite states. theta is a double
