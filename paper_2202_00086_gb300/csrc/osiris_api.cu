@@ -667,11 +667,11 @@ struct osiris_batch_plan {
   int32_t max_requests = 0;
   int32_t spacetime = OSIRIS_SPACETIME_KERR;
   int block = 0;
-  // the kernels of a small and of a large launch, each with its full grid
+  // the kernels of a tiny, a small and a large launch, each with its full grid
   struct {
     const void* fn;
     int64_t full_grid;
-  } variant[2] = {};
+  } variant[3] = {};
   ReqDev* staging = nullptr;    // pinned host copy of the request table
   ReqDev* dev_table = nullptr;  // inside opts.workspace
   cudaEvent_t copied = nullptr;  // recorded by the graph once the table is uploaded
@@ -691,6 +691,10 @@ void release(osiris_batch_plan* p) {
   if (p->copied) cudaEventDestroy(p->copied);
   if (p->staging) cudaFreeHost(p->staging);
   delete p;
+}
+
+Kernel round_kind(int64_t rays) {
+  return rays < osiris_impl::kTinyRound ? Kernel::kTinyRound : Kernel::kPersistent;
 }
 
 // Record upload -> event -> queue reset -> kernel on a private stream.
@@ -771,9 +775,9 @@ int osiris_batch_plan_create(osiris_batch_plan** out, int32_t max_requests, int3
                                            osiris_impl::kQueueBytes);
   p->block = block_of(&p->opts);
   int rc = OSIRIS_OK;
-  for (int k = 0; k < 2 && rc == OSIRIS_OK; ++k) {
-    p->variant[k].fn = kernel_of(&p->opts, Kernel::kPersistent, spacetime,
-                                 k ? INT64_MAX : osiris_impl::kTinyBatch);
+  const int64_t rays[3] = {1, osiris_impl::kTinyRound, INT64_MAX};
+  for (int k = 0; k < 3 && rc == OSIRIS_OK; ++k) {
+    p->variant[k].fn = kernel_of(&p->opts, round_kind(rays[k]), spacetime, rays[k]);
     rc = full_grid(&p->opts, p->variant[k].fn, &p->variant[k].full_grid);
   }
   if (rc == OSIRIS_OK &&
@@ -819,8 +823,10 @@ int osiris_batch_plan_launch(osiris_batch_plan* p, const osiris_request* reqs, i
   set_granularity(args, &p->opts);
   const int64_t per_block = static_cast<int64_t>(p->block) * args.rays_per_lane;
   int64_t grid = (total + per_block - 1) / per_block;
-  const void* fn = kernel_of(&p->opts, Kernel::kPersistent, p->spacetime, total);
-  const int64_t most = p->variant[fn == p->variant[0].fn ? 0 : 1].full_grid;
+  const void* fn = kernel_of(&p->opts, round_kind(total), p->spacetime, total);
+  int64_t most = p->variant[0].full_grid;
+  for (const auto& v : p->variant)
+    if (v.fn == fn) most = v.full_grid;
   if (grid > most) grid = most;
   cudaKernelNodeParams k = p->kernel;
   k.func = const_cast<void*>(fn);

@@ -52,15 +52,17 @@ namespace osiris_impl {
 constexpr int64_t kLargeLaunch = 7 * 152 * 256 / 2;
 constexpr int kLargeRegs = 128;
 
+template <bool kTiny>
 struct KerrDF {
+  static constexpr bool kTinyRounds = kTiny;
   using Ray = RayDF;
-  static constexpr int kMaxRegs = kLargeRegs;
+  static constexpr int kMaxRegs = kTiny ? 80 : kLargeRegs;
   static constexpr bool kFusedR2 = true;
   static __device__ __forceinline__ Ray ray(const RayK& K) { return to_df(K); }
   static __device__ __forceinline__ void rhs(const Ray& K, df r, df th, df pr, df pth, df& dr,
                                              df& dth, df& dph, df& dpr, df& dpth,
                                              float& twoH) {
-    rhs_df(K, r, th, pr, pth, dr, dth, dph, dpr, dpth, twoH);
+    rhs_df<kTiny>(K, r, th, pr, pth, dr, dth, dph, dpr, dpth, twoH);
   }
   static constexpr bool kTrackH = true;
   static constexpr bool kF32Stages = false;
@@ -73,15 +75,17 @@ struct KerrDF {
   }
 };
 
+template <bool kTiny>
 struct QMetricDF {
+  static constexpr bool kTinyRounds = kTiny;
   using Ray = RayQDF;
-  static constexpr int kMaxRegs = kLargeRegs;
+  static constexpr int kMaxRegs = kTiny ? 80 : kLargeRegs;
   static constexpr bool kFusedR2 = true;
   static __device__ __forceinline__ Ray ray(const RayK& K) { return to_qdf(K); }
   static __device__ __forceinline__ void rhs(const Ray& K, df r, df th, df pr, df pth, df& dr,
                                              df& dth, df& dph, df& dpr, df& dpth,
                                              float& twoH) {
-    rhs_q_df(K, r, th, pr, pth, dr, dth, dph, dpr, dpth, twoH);
+    rhs_q_df<kTiny>(K, r, th, pr, pth, dr, dth, dph, dpr, dpth, twoH);
   }
   static constexpr bool kTrackH = true;
   static constexpr bool kF32Stages = false;
@@ -112,20 +116,23 @@ static const void* df64_kernel(Kernel kind) {
                                      : (const void*)trace_df64_plain<Met, INTEG, kLarge>;
 }
 
-template <class Met>
-static const void* df64_kernel(Kernel kind, int integrator, bool large) {
-  if (integrator == OSIRIS_RKDP45)
-    return large ? df64_kernel<Met, OSIRIS_RKDP45, true>(kind)
-                 : df64_kernel<Met, OSIRIS_RKDP45, false>(kind);
-  return large ? df64_kernel<Met, OSIRIS_RKCK45, true>(kind)
-               : df64_kernel<Met, OSIRIS_RKCK45, false>(kind);
+template <template <bool> class Met, int INTEG>
+static const void* df64_kernel(Kernel kind, int64_t rays) {
+  if (kind == Kernel::kTinyRound)
+    return (const void*)trace_df64_persistent<Met<true>, INTEG, true>;
+  return rays >= kLargeLaunch ? df64_kernel<Met<false>, INTEG, true>(kind)
+                              : df64_kernel<Met<false>, INTEG, false>(kind);
+}
+
+template <template <bool> class Met>
+static const void* df64_kernel(Kernel kind, int integrator, int64_t rays) {
+  return integrator == OSIRIS_RKDP45 ? df64_kernel<Met, OSIRIS_RKDP45>(kind, rays)
+                                     : df64_kernel<Met, OSIRIS_RKCK45>(kind, rays);
 }
 
 const void* trace_kernel_df64(Kernel kind, int integrator, int spacetime, int64_t rays) {
-  const bool large =
-      rays >= kLargeLaunch || (kind == Kernel::kPersistent && rays < kTinyBatch);
-  return spacetime == OSIRIS_SPACETIME_QMETRIC ? df64_kernel<QMetricDF>(kind, integrator, large)
-                                               : df64_kernel<KerrDF>(kind, integrator, large);
+  return spacetime == OSIRIS_SPACETIME_QMETRIC ? df64_kernel<QMetricDF>(kind, integrator, rays)
+                                               : df64_kernel<KerrDF>(kind, integrator, rays);
 }
 
 }  // namespace osiris_impl

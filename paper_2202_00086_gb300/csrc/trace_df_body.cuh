@@ -119,7 +119,7 @@ __device__ __forceinline__ void trace_body_df(const KernelArgs& A) {
   int kind = 0, side = 0, iters = 0;
   double lo = 0, hi = 0, h_try = 0;  // surface location: the step-length bracket
   df h_try_df = mk(0.0f, 0.0f);       // h_try as the stepper takes it
-  float h_step = 0.0f;                // length of the last accepted step
+  float h_step = 0.0f;                // length of the step that crossed the equator, and its end yE
   float flo = 0.0f, fhi = 0.0f;
   StateDF yF, yE;
   std::conditional_t<Met::kF32Stages, LaneCacheF32<INTEG>, LaneCacheDF<INTEG>> LC;
@@ -280,21 +280,23 @@ __device__ __forceinline__ void trace_body_df(const KernelArgs& A) {
         finish(OSIRIS_STATUS_ERROR, y);
         continue;
       }
+      // step-size controller: min(5, max(0.2, 0.9 err^-1/5)) after an accepted
+      // attempt, max(0.1, 0.9 err^-1/4) after a rejected one; one power for
+      // both, ahead of the branch that lanes of a warp take differently
+      const float factor = 0.9f * exp2f((ok ? -0.2f : -0.25f) * log2f(err));
+      h = hs_f * (ok ? fminf(5.0f, fmaxf(0.2f, factor)) : fmaxf(0.1f, factor));
       if (ok) {
         ++n_acc;
-        const float grow = fminf(5.0f, fmaxf(0.2f, 0.9f * exp2f(-0.2f * log2f(err))));
-        h = hs_f * grow;
-        h_step = hs_f;
-        yE = o;
         if (I.disk && ((df_side(y.th) > 0.0f && df_side(o.th) <= 0.0f) ||
-                       (df_side(y.th) < 0.0f && df_side(o.th) >= 0.0f)))
-          begin_locate(SURF_EQUATOR, h_step, o);
-        else
-          after_accept(h_step, o, true);
+                       (df_side(y.th) < 0.0f && df_side(o.th) >= 0.0f))) {
+          h_step = hs_f;
+          yE = o;
+          begin_locate(SURF_EQUATOR, hs_f, o);
+        } else {
+          after_accept(hs_f, o, true);
+        }
       } else {
         ++n_rej;
-        const float shrink = fmaxf(0.1f, 0.9f * exp2f(-0.25f * log2f(err)));
-        h = hs_f * shrink;
         if ((int64_t)(n_acc + n_rej) >= I.max_steps) finish(OSIRIS_STATUS_MAXSTEP, y);
       }
     } else {  // MODE_LOCATE: Illinois-modified regula falsi on the step length

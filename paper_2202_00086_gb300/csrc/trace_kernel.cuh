@@ -441,22 +441,22 @@ __device__ __forceinline__ void trace_body(const KernelArgs& A) {
         err_component(y.pr, o.pr, d.pr, tol, ok, err);
         err_component(y.pth, o.pth, d.pth, tol, ok, err);
       }
+      // step-size controller (FP32 is enough to size the next step):
+      // min(5, max(0.2, 0.9 err^-1/5)) after an accepted attempt, max(0.1,
+      // 0.9 err^-1/4) after a rejected one
+      const float factor = 0.9f * exp2f((ok ? -0.2f : -0.25f) * log2f(err));
+      h = hs * float_to_double(ok ? fminf(5.0f, fmaxf(0.2f, factor)) : fmaxf(0.1f, factor));
       if (ok) {
         ++n_acc;
-        // step-size controller (FP32 is enough to size the next step):
-        // min(5, max(0.2, 0.9 err^-1/5))
-        const float grow = fminf(5.0f, fmaxf(0.2f, 0.9f * exp2f(-0.2f * log2f(err))));
-        h = hs * float_to_double(grow);
-        h_step = hs;
-        yE = o;
-        if (disk && crosses_equator(y, o))
+        if (disk && crosses_equator(y, o)) {
+          h_step = hs;
+          yE = o;
           begin_locate(SURF_EQUATOR, hs, o);
-        else
+        } else {
           after_accept(hs, o, true);
+        }
       } else {
         ++n_rej;
-        const float shrink = fmaxf(0.1f, 0.9f * exp2f(-0.25f * log2f(err)));
-        h = hs * float_to_double(shrink);
         if ((int64_t)(n_acc + n_rej) >= max_steps) finish(OSIRIS_STATUS_MAXSTEP, y);
       }
     } else {  // MODE_LOCATE: Illinois-modified regula falsi on the step length
