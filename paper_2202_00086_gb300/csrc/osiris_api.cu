@@ -667,7 +667,8 @@ struct osiris_batch_plan {
   int32_t max_requests = 0;
   int32_t spacetime = OSIRIS_SPACETIME_KERR;
   int block = 0;
-  // the kernels of a tiny, a small and a large launch, each with its full grid
+  // the kernels that this plan has launched (of a tiny, a small and a large
+  // round), each with its full grid
   struct {
     const void* fn;
     int64_t full_grid;
@@ -722,7 +723,8 @@ int record_plan(osiris_batch_plan* p) {
                       cudaMemcpyHostToDevice, cs) != cudaSuccess ||
       cudaEventRecordWithFlags(p->copied, cs, cudaEventRecordExternal) != cudaSuccess ||
       cudaMemsetAsync(args.queue, 0, sizeof(unsigned long long), cs) != cudaSuccess ||
-      launch_kernel(p->variant[0].fn, args, 1, p->block, cs) != OSIRIS_OK)
+      launch_kernel(kernel_of(&p->opts, Kernel::kPersistent, p->spacetime, INT64_MAX), args, 1,
+                    p->block, cs) != OSIRIS_OK)
     rc = OSIRIS_ECUDA;
   cudaGraph_t g = nullptr;
   if (cudaStreamEndCapture(cs, &g) != cudaSuccess) rc = OSIRIS_ECUDA;
@@ -775,11 +777,6 @@ int osiris_batch_plan_create(osiris_batch_plan** out, int32_t max_requests, int3
                                            osiris_impl::kQueueBytes);
   p->block = block_of(&p->opts);
   int rc = OSIRIS_OK;
-  const int64_t rays[3] = {1, osiris_impl::kTinyRound, INT64_MAX};
-  for (int k = 0; k < 3 && rc == OSIRIS_OK; ++k) {
-    p->variant[k].fn = kernel_of(&p->opts, round_kind(rays[k]), spacetime, rays[k]);
-    rc = full_grid(&p->opts, p->variant[k].fn, &p->variant[k].full_grid);
-  }
   if (rc == OSIRIS_OK &&
       cudaMallocHost(&p->staging, sizeof(ReqDev) * static_cast<size_t>(max_requests)) !=
           cudaSuccess) {
@@ -824,9 +821,17 @@ int osiris_batch_plan_launch(osiris_batch_plan* p, const osiris_request* reqs, i
   const int64_t per_block = static_cast<int64_t>(p->block) * args.rays_per_lane;
   int64_t grid = (total + per_block - 1) / per_block;
   const void* fn = kernel_of(&p->opts, round_kind(total), p->spacetime, total);
-  int64_t most = p->variant[0].full_grid;
-  for (const auto& v : p->variant)
-    if (v.fn == fn) most = v.full_grid;
+  int64_t most = 0;
+  for (auto& v : p->variant) {
+    if (v.fn == nullptr) {  // the plan's first round of this size
+      if (int rc = full_grid(&p->opts, fn, &v.full_grid)) return rc;
+      v.fn = fn;
+    }
+    if (v.fn == fn) {
+      most = v.full_grid;
+      break;
+    }
+  }
   if (grid > most) grid = most;
   cudaKernelNodeParams k = p->kernel;
   k.func = const_cast<void*>(fn);
