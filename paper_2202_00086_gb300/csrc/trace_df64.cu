@@ -33,23 +33,26 @@ namespace osiris_impl {
 // Metric policies of the double-float kernels: the ray constants, the
 // evaluation, and the register cap.
 //
-// Two variants, chosen by the launch's rays. Large launches: 128 registers, so
-// that four blocks of 128 threads (16 warps) are resident per SM: the
-// double-float dependency chains need the extra warps more than they lose to
-// the spilled values, which stay in L1 as long as no shared memory is
-// reserved (12 x 1024^2 Kerr set, Mrays/s, Cash-Karp: 168 registers (three
-// blocks) 14.4, 128: 15.5, 112: 15.4, 96: 15.3, 80: 14.7). Small launches have
-// one or two warps per SM sub-partition and last as long as their longest
-// chains: no cap (201-231 registers, two blocks per SM), nothing spilled. 128
-// registers / no cap, ms:
-//   Kerr render  32^2  5.2 / 3.3     100^2  6.3 / 4.0     160^2  7.4 / 5.2
-//               256^2  7.8 / 7.1     360^2 11.9 / 10.1    512^2 18.1 / 18.3
-//   disk        100^2  4.3 / 2.9     256^2  5.7 / 5.3     400^2  9.3 / 9.5
-//   q-metric     64^2  9.0 / 6.3     300^2 17.7 / 15.4    600^2 38.3 / 42.5
-//   Dormand-Prince render  64^2  6.3 / 4.2    400^2 14.1 / 13.4    800^2 39.2 / 43.8
-//   particles    5,000  1.1 / 0.75  100,000  2.55 / 2.55
-// The line lies at 3.5 times the lanes of the uncapped kernels in flight.
-constexpr int64_t kLargeLaunch = 7 * 152 * 256 / 2;
+// Two variants, chosen by the launch's rays. Small launches have one or two
+// warps per SM sub-partition and last as long as their longest chains: no cap
+// (203-234 registers, two blocks of 128 threads per SM), nothing spilled.
+// Large launches: 128 registers, so that four blocks are resident per SM: the
+// double-float dependency chains gain more from the extra warps than they lose
+// to the spilled values, which stay in L1 as long as no shared memory is
+// reserved. 128 registers / 168 (three blocks) / no cap, ms:
+//   Kerr render  100^2  4.7 / - / 3.0      360^2   9.7 / 9.2 / 8.3    512^2  15.4 / 15.1 / 14.0
+//                640^2 21.9 / 21.9 / 20.6  800^2  31.0 / 30.9 / 30.7  2048^2 184.6 / 185.9 / 187.4
+//   disk         400^2  8.5 / 8.1 / 8.0    600^2  15.5 / 15.4 / 15.2  2048^2 153.7 / 155.3 / 158.2
+//   six renders  200^2 15.9 / 15.9 / 14.9  400^2  51.2 / 50.4 / 50.8  800^2 189.0 / 189.1 / 194.0
+//   particles    100,000  2.33 / 1.99 / 1.83      400,000  5.74 / 5.68 / 5.88
+//   Dormand-Prince render     400^2 12.4 / 13.2 / 10.9   1024^2 56.3 / 57.9 / 56.7
+//   q-metric     300^2 15.8 / 15.5 / 13.5  512^2  27.3 / 28.3 / 27.0  600^2  34.3 / 35.6 / 34.5
+//               1024^2 82.4 / 87.2 / 88.0  six 200^2 27.1 / 27.6 / 27.0
+// The lines lie at 10 (Kerr) and 8 (q-metric) times the lanes that the uncapped
+// kernels keep in flight (256 on each of 152 SMs), where the first kind of
+// launch gets no slower by the cap (Kerr particles, q-metric renders).
+constexpr int64_t kLargeLaunchKerr = 10 * 152 * 256;
+constexpr int64_t kLargeLaunchQ = 8 * 152 * 256;
 constexpr int kLargeRegs = 128;
 
 template <bool kTiny>
@@ -117,22 +120,23 @@ static const void* df64_kernel(Kernel kind) {
 }
 
 template <template <bool> class Met, int INTEG>
-static const void* df64_kernel(Kernel kind, int64_t rays) {
+static const void* df64_kernel(Kernel kind, int64_t rays, int64_t line) {
   if (kind == Kernel::kTinyRound)
     return (const void*)trace_df64_persistent<Met<true>, INTEG, true>;
-  return rays >= kLargeLaunch ? df64_kernel<Met<false>, INTEG, true>(kind)
-                              : df64_kernel<Met<false>, INTEG, false>(kind);
+  return rays >= line ? df64_kernel<Met<false>, INTEG, true>(kind)
+                      : df64_kernel<Met<false>, INTEG, false>(kind);
 }
 
 template <template <bool> class Met>
-static const void* df64_kernel(Kernel kind, int integrator, int64_t rays) {
-  return integrator == OSIRIS_RKDP45 ? df64_kernel<Met, OSIRIS_RKDP45>(kind, rays)
-                                     : df64_kernel<Met, OSIRIS_RKCK45>(kind, rays);
+static const void* df64_kernel(Kernel kind, int integrator, int64_t rays, int64_t line) {
+  return integrator == OSIRIS_RKDP45 ? df64_kernel<Met, OSIRIS_RKDP45>(kind, rays, line)
+                                     : df64_kernel<Met, OSIRIS_RKCK45>(kind, rays, line);
 }
 
 const void* trace_kernel_df64(Kernel kind, int integrator, int spacetime, int64_t rays) {
-  return spacetime == OSIRIS_SPACETIME_QMETRIC ? df64_kernel<QMetricDF>(kind, integrator, rays)
-                                               : df64_kernel<KerrDF>(kind, integrator, rays);
+  return spacetime == OSIRIS_SPACETIME_QMETRIC
+             ? df64_kernel<QMetricDF>(kind, integrator, rays, kLargeLaunchQ)
+             : df64_kernel<KerrDF>(kind, integrator, rays, kLargeLaunchKerr);
 }
 
 }  // namespace osiris_impl

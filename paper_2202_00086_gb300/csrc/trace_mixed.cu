@@ -32,30 +32,31 @@
 
 namespace osiris_impl {
 
-// Registers. Large launches are bound by issue slots and gain from warps that
-// hide the dependent FP32 chains: 80 registers (six blocks of 128 threads per
-// SM) for Kerr, 128 (four) for the q-metric. Measured at tol 1e-8 on the
-// 12 x 1024^2 Kerr set (Mrays/s, Cash-Karp, refill at 32 idle lanes): 96
-// registers 160.9, 80: 162.3, 72: 154.7, 64: 153.0; on six 500^2 q-metric
-// renders in one launch (ms) 56 registers 13.8, 80: 14.6, 104: 14.5, 128: 12.7,
-// no cap 13.5, on a 1024^2 render 9.45 / 9.47 / 10.1 / 9.17 / 9.9. Small
-// launches last as long as their longest chains: no cap (145-160 registers,
-// three blocks per SM), nothing spilled. 80 / no cap, in ms, for Kerr:
-//   render     32^2  0.80 / 0.62    256^2  1.13 / 0.99    512^2  2.37 / 2.29
-//             800^2  4.32 / 4.58
-//   disk      200^2  1.08 / 0.89    500^2  1.85 / 1.82    900^2  4.51 / 4.91
-//   six renders in one launch  100^2  1.33 / 1.12    200^2  2.51 / 2.52    400^2  7.2 / 7.6
-//   Dormand-Prince render      200^2  1.13 / 0.89    400^2  1.76 / 1.66    800^2  4.46 / 4.81
-// and 128 / no cap for the q-metric: 100^2 0.89 / 0.82, 300^2 1.68 / 1.60, 600^2
-// 3.69 / 3.94, six 200^2 renders 2.89 / 2.93. The lines lie at 5 and 2.5 times
-// 256 lanes on each of 152 SMs.
-constexpr int64_t kLargeLaunchKerr = 5 * 152 * 256;
-constexpr int64_t kLargeLaunchQ = 5 * 152 * 256 / 2;
+// Registers. Small launches last as long as their longest chains: no cap
+// (three blocks of 128 threads per SM), nothing spilled. Large launches are
+// bound by issue slots and gain from warps that hide the dependent FP32 chains:
+// 96 registers (five blocks) for Kerr, 128 (four) for the q-metric (earlier
+// sweeps: Kerr 72 and 64 slower than 80, q-metric 56 and 80 slower than 128).
+// Kerr, 80 / 96 / no cap, ms at tol 1e-8:
+//   render   360^2  1.35 / 1.37 / 1.21    512^2  2.10 / 2.02 / 1.96    640^2  3.01 / 2.93 / 2.84
+//            800^2  3.92 / 3.91 / 4.01   1024^2  6.19 / 6.17 / 6.40   2048^2 22.83 / 22.78 / 23.44
+//   disk     400^2  1.21 / 1.17 / 1.14    600^2  2.11 / 2.10 / 2.17   2048^2 19.46 / 19.54 / 20.85
+//   six renders in one launch  200^2  2.20 / 2.17 / 2.13   400^2  6.59 / 6.52 / 6.62
+//                              800^2 23.57 / 23.13 / 23.77
+//   particles  100,000  0.366 / 0.349 / 0.326    400,000  0.960 / 0.951 / 0.977
+//   Dormand-Prince render      400^2  1.56 / 1.55 / 1.45   1024^2 6.50 / 6.53 / 6.69
+// q-metric, 128 / 104 / no cap:
+//   render   300^2  1.46 / 1.51 / 1.27    400^2  1.91 / 2.01 / 1.79    512^2  2.64 / 2.86 / 2.67
+//            600^2  3.29 / 3.62 / 3.34   1024^2  8.17 / 8.91 / 8.46
+//   six renders in one launch  200^2  2.55 / 2.68 / 2.52   500^2 11.5 / 12.4 / 11.9
+// The lines lie at 8 and 5 times 256 lanes on each of 152 SMs.
+constexpr int64_t kLargeLaunchKerr = 8 * 152 * 256;
+constexpr int64_t kLargeLaunchQ = 5 * 152 * 256;
 
 template <bool kTiny>
 struct KerrMixed {
   using Ray = RayF32;
-  static constexpr int kMaxRegs = 80;
+  static constexpr int kMaxRegs = kTiny ? 80 : 96;
   static constexpr bool kFusedR2 = false;
   static constexpr bool kTrackH = false;
   static constexpr bool kF32Stages = true;
