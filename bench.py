@@ -55,18 +55,17 @@ LOOSE_TOL = 1e-8  # the served stream's looser tolerance, where MIXED is meant t
 FP64_TRAFFIC_BYTES_PER_LAUNCH = 575.78e6
 # FP32-pipe (FMA heavy + lite) thread instructions, and warp instructions of
 # every pipe, per double-float Cash-Karp attempt on the Kerr set: ncu capture
-# of trace_df64_persistent on the 12 renders at 256x256 (3.3475e10 FMA-pipe
-# warp instructions x 28.71 active lanes, and 4.050e10 warp instructions, over
-# 2.7322e8 attempts), profiles/trace_df64_persistent_kerr12x256_ncu.md.
-DF64_FP32_INST_PER_ATTEMPT = 3518
-DF64_WARP_INST_PER_ATTEMPT = 148.2
+# of trace_df64_persistent on the 12 renders at 256x256 (3.3035e10 FMA-pipe
+# warp instructions x 28.97 active lanes, and 3.843e10 warp instructions, over
+# 2.7322e8 attempts), profiles/trace_persistent_counters.md.
+DF64_FP32_INST_PER_ATTEMPT = 3503
+DF64_WARP_INST_PER_ATTEMPT = 140.7
 # The same for the MIXED kernel (FP32 evaluations, FP32 stage sums) at tol
 # 1e-8: ncu capture of trace_mixed_persistent on the 12 renders at 256x256
-# (3.6500e9 FMA-pipe warp instructions x 25.19 active lanes, and 5.5962e9 warp
-# instructions, over 1.4642e8 attempts),
-# profiles/trace_mixed_persistent_kerr12x256_ncu.md.
-MIXED_FP32_INST_PER_ATTEMPT = 628
-MIXED_WARP_INST_PER_ATTEMPT = 38.22
+# (3.5845e9 FMA-pipe warp instructions x 25.87 active lanes, and 5.3165e9 warp
+# instructions, over 1.4642e8 attempts), profiles/trace_persistent_counters.md.
+MIXED_FP32_INST_PER_ATTEMPT = 633
+MIXED_WARP_INST_PER_ATTEMPT = 36.31
 
 
 def fp32_roofline(probe, inst_per_attempt, warp_inst_per_attempt, attempts, seconds):

@@ -95,7 +95,7 @@ typedef struct {
                               |y5 - y4| / (tol (1 + max(|y_n|, |y_n+1|)))), > 0 */
     int64_t max_steps;     /* cap on accepted + rejected steps per ray, >= 1 */
     int32_t precision;     /* OSIRIS_FP64, OSIRIS_MIXED or OSIRIS_DF64 */
-    int32_t persistent;    /* 0: one ray per thread; 1: persistent grid that
+    int32_t persistent;    /* 0: plain launch, no workspace; 1: persistent grid that
                               refills lanes from a device ray queue (needs
                               workspace) */
     double r_cap_factor;   /* captured when r < r_cap_factor * r_H, > 1 */
@@ -114,9 +114,9 @@ typedef struct {
     size_t workspace_bytes;
     int32_t integrator;    /* OSIRIS_RKCK45 (default) or OSIRIS_RKDP45 */
     int32_t rays_per_lane; /* rays a lane takes at once, 0..64 (0 = 1): a plain
-                              launch gives each thread this many consecutive
-                              pixels; a persistent grid claims this many per
-                              idle lane with each queue atomic */
+                              launch deals out this many consecutive pixels
+                              per thread at a time; a persistent grid claims
+                              this many per idle lane with each queue atomic */
     int32_t refill_lanes;  /* persistent grid, 0..32 (0 = library default: 4,
                               32 in OSIRIS_MIXED): a
                               warp whose other lanes are still integrating

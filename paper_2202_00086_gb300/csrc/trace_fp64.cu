@@ -120,12 +120,13 @@ struct StepperFP64<OSIRIS_RKDP45, Met, kLarge> {
 // ~195, two blocks of 128 threads per SM). Large ones are bound by the FP64
 // unit: sums on the integer pipes where they are cheap there (ArithFast<true>),
 // and four blocks per SM to hide the longer chains. Small / large variant, ms:
-//   Cash-Karp   render    64^2  13.7 / 16.2     320^2  32.8 / 31.8
-//                        384^2  44.1 / 42.9     512^2  64.4 / 58.9
-//                        768^2   131 / 110      twelve 400^2 in a batch 382 / 347
-//   particles  30,000     2.7 / 2.9             500,000  33.8 / 30.0
-//   Dormand-Prince disk  512 x 256  30.0 / 33.4     600 x 300  35.0 / 35.0
-//                        800 x 400  56.2 / 54.1    1024 x 512  89.3 / 80.2
+//   Cash-Karp   render    32^2  12.3 / 15.3     256^2  24.7 / 29.7
+//                        360^2  35.2 / 36.3     512^2  57.7 / 56.7
+//                        800^2   128 / 110
+//               six in a batch  100^2 23.7 / 26.6    200^2 63.1 / 60.0    400^2  207 / 184
+//               disk     256^2  18.7 / 20.4     400^2  30.3 / 29.5     600^2  61.3 / 54.0
+//   particles   5,000  2.1 / 2.6     100,000  6.6 / 7.0     400,000  21.7 / 20.1
+//   Dormand-Prince render 64^2  14.0 / 17.1     400^2  42.6 / 43.1     800^2   135 / 117
 // The line lies at five times the lanes that the small variant keeps in
 // flight. Caps of 168 registers (three blocks) with either sums lie between
 // the two. The q-metric has the small variant only: twice the integer work
