@@ -38,7 +38,8 @@ extern "C" {
 #define OSIRIS_ETIMEOUT (-4) /* a bounded wait ran out */
 
 /* ---- per-ray status (the fate of the backward ray; Sec. 4.1, Sec. 5) ---- */
-#define OSIRIS_STATUS_NONE 0     /* not traced */
+#define OSIRIS_STATUS_NONE 0     /* not traced (plain FP64 and DF64 launches set every
+                                    ray's status to it first, on the stream) */
 #define OSIRIS_STATUS_CAPTURED 1 /* reached r < r_cap_factor * r_H */
 #define OSIRIS_STATUS_ESCAPED 2  /* reached the celestial sphere r > r_esc_factor * r_obs */
 #define OSIRIS_STATUS_DISK 3     /* hit the equatorial disk r_in <= r <= r_out */
@@ -83,6 +84,9 @@ extern "C" {
                                        (check code << 56) | ray index; codes 1 ray index
                                        outside the launch, 2 request index, 3 ray outside
                                        its request's range, 4 pixel / state index */
+#define OSIRIS_STAT_GAVE_UP 15      /* warps of a plain FP64 or DF64 launch that waited in
+                                       vain for more rays (a second or more): rays may then
+                                       be left untraced, with OSIRIS_STATUS_NONE */
 #define OSIRIS_STATS_LEN 16
 
 /* Opaque camera: space-time, observer and image plane. Host memory only. */

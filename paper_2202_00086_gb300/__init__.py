@@ -446,6 +446,7 @@ def decode_stats(stats):
     out = {name: int(v[k]) for k, name in enumerate(STAT_NAMES)}
     out["max_abs_H"] = ctypes.cast(ctypes.pointer(ctypes.c_int64(v[11])),
                                    _P(_d)).contents.value
+    out["gave_up"] = int(v[15])
     return out
 
 

@@ -230,6 +230,11 @@ int launch(KernelArgs& args, const osiris_trace_opts* o, void* stream) {
                        : per_block;
       args.refill_lanes = args.single.explicit_states ? kRefillLanesStates : 32;
       grid = (args.total_rays + args.chunk - 1) / args.chunk;
+      // a ray that no block traces must not pass for a traced one
+      if (args.single.out.status &&
+          cudaMemsetAsync(args.single.out.status, OSIRIS_STATUS_NONE, args.total_rays, s) !=
+              cudaSuccess)
+        return OSIRIS_ECUDA;
     }
     return launch_kernel(kernel_of(o, Kernel::kPlain, spacetime, args.total_rays), args, grid,
                          block, s);

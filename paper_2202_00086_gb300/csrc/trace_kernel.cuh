@@ -398,8 +398,8 @@ __device__ __forceinline__ void trace_body(const KernelArgs& A) {
       if (steal_refill(A, (mode == MODE_IDLE) && !drained, busy, first, over)) start_ray(first);
       drained |= over;
       if (!__any_sync(FULL, mode != MODE_IDLE)) {
-        if (drained || ++turns_without > kStealPatience) break;
-        continue;
+        if (steal_waits(A, drained, turns_without)) continue;
+        break;
       }
       turns_without = 0;
     }

@@ -60,11 +60,13 @@ __device__ __forceinline__ void steal_request() {
   // the answer to the previous request has been read before this one is written
   asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], 16;" ::"r"(bar) : "memory");
+#ifndef OSIRIS_STEAL_MUTE  // test builds: no request is sent, so that no answer ever comes
   asm volatile(
       "clusterlaunchcontrol.try_cancel.async.shared::cta.mbarrier::complete_tx::bytes.b128 "
       "[%0], [%1];" ::"r"(shared_address(&P.response)),
       "r"(bar)
       : "memory");
+#endif
   P.pending = 1;
 }
 
@@ -159,8 +161,25 @@ __device__ __forceinline__ int steal_refill(const KernelArgs& A, bool need, bool
   return 1;
 }
 
-// Turns of a warp without any ray after which it gives up (about a second: an
-// answer takes about a microsecond).
-constexpr unsigned kStealPatience = 1u << 24;
+// Turns in a row that a warp without any ray waits for more of them. It waits
+// only while the block's request is unanswered, about a microsecond, and a turn
+// takes some hundred cycles, so 2^24 of them are a second or more. (A count of
+// turns, not a time: it stands still while the GPU runs something else.)
+#ifndef OSIRIS_STEAL_PATIENCE
+#define OSIRIS_STEAL_PATIENCE (1u << 24)
+#endif
+constexpr unsigned kStealPatience = OSIRIS_STEAL_PATIENCE;
+
+// Whether a warp without any ray asks again. It leaves once the block gets no
+// more rays (`drained`), with no request outstanding then, or when its wait has
+// run out. That is counted in the stats, and the rays that such a block may
+// have taken over and not traced keep the OSIRIS_STATUS_NONE that the launch
+// starts with.
+__device__ __forceinline__ bool steal_waits(const KernelArgs& A, bool drained, unsigned& turns) {
+  if (drained) return false;
+  if (++turns <= kStealPatience) return true;
+  if ((threadIdx.x & 31) == 0 && A.stats) atomicAdd(A.stats + OSIRIS_STAT_GAVE_UP, 1ull);
+  return false;
+}
 
 }  // namespace osiris_impl
