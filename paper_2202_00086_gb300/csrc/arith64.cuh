@@ -22,7 +22,7 @@
 // do not test each product: they test that the factors which are not products
 // themselves lie in [2^-63, 2^65) (window(), two integer instructions a
 // value), from which the range of every product follows; an attempt that
-// fails the test (bad()) is done again with plain FP64 instructions. Factors
+// fails the test (bad()) stops and is done with plain FP64 instructions. Factors
 // that are zero in ordinary use (the spin of Schwarzschild, L of the middle
 // column, p_theta of the middle row) are never given to soft_mul; those that a
 // soft_mul0 takes are tested with window0().
@@ -158,8 +158,10 @@ struct ArithPlain {
     return s + float_to_double0(f);
   }
   __device__ __forceinline__ double minus_two(double r) const { return r - 2.0; }
+  __device__ __forceinline__ bool bad() const { return false; }
   __device__ __forceinline__ void window(double) const {}
   __device__ __forceinline__ void window0(double) const {}
+  __device__ __forceinline__ void wide0(double) const {}
 };
 
 // a + c on the FP64 unit where a sum on the integer pipes does not apply. Out
@@ -214,6 +216,12 @@ struct ArithFast {
   // the same, or zero
   __device__ __forceinline__ void window0(double x) {
     const unsigned v = ((unsigned)(bits_of(x) >> 32) + 0x04000000u) ^ 0x40000000u;
+    range |= (bits_of(x) << 1) == 0 ? 0u : v;
+  }
+  // |x| in [2^-511, 2^513) or zero, for a factor whose product enters sums only:
+  // biased exponents 512..1535, so that 512 more have the leading bit set
+  __device__ __forceinline__ void wide0(double x) {
+    const unsigned v = ~((unsigned)(bits_of(x) >> 32) + 0x20000000u) & 0x40000000u;
     range |= (bits_of(x) << 1) == 0 ? 0u : v;
   }
   __device__ __forceinline__ bool bad() const { return (range & 0x78000000u) != 0; }
