@@ -201,7 +201,6 @@ __device__ __forceinline__ float flip_sign(float x, unsigned sign) {
   return __uint_as_float(__float_as_uint(x) ^ sign);
 }
 
-template <bool kBranches = false>  // kBranches: see kTinyRound (osiris_internal.h)
 __device__ __forceinline__ void df_sincos(df x, df& s, df& c) {
   using namespace dfc;
   const float k = rintf(x.hi * 0.636619772367581343f);
@@ -235,22 +234,6 @@ __device__ __forceinline__ void df_sincos(df x, df& s, df& c) {
   qc = df_add_to_f_u(-0.5f, df_mul(u, qc));
   const df ct = df_add_to_f_u(1.0f, df_mul(u, qc));
   const int q = (int)k;
-  if (kBranches) {
-    if ((q & 3) == 0) {
-      s = st;
-      c = ct;
-    } else if ((q & 3) == 1) {
-      s = ct;
-      c = df_neg(st);
-    } else if ((q & 3) == 2) {
-      s = df_neg(st);
-      c = df_neg(ct);
-    } else {
-      s = df_neg(ct);
-      c = st;
-    }
-    return;
-  }
   const bool odd = (q & 1) != 0;
   const df s0 = mk(odd ? ct.hi : st.hi, odd ? ct.lo : st.lo);
   const df c0 = mk(odd ? st.hi : ct.hi, odd ? st.lo : ct.lo);

@@ -672,12 +672,12 @@ struct osiris_batch_plan {
   int32_t max_requests = 0;
   int32_t spacetime = OSIRIS_SPACETIME_KERR;
   int block = 0;
-  // the kernels that this plan has launched (of a tiny, a small and a large
-  // round), each with its full grid
+  // the kernels that this plan has launched (of a small and a large round),
+  // each with its full grid
   struct {
     const void* fn;
     int64_t full_grid;
-  } variant[3] = {};
+  } variant[2] = {};
   ReqDev* staging = nullptr;    // pinned host copy of the request table
   ReqDev* dev_table = nullptr;  // inside opts.workspace
   cudaEvent_t copied = nullptr;  // recorded by the graph once the table is uploaded
@@ -697,10 +697,6 @@ void release(osiris_batch_plan* p) {
   if (p->copied) cudaEventDestroy(p->copied);
   if (p->staging) cudaFreeHost(p->staging);
   delete p;
-}
-
-Kernel round_kind(int64_t rays) {
-  return rays < osiris_impl::kTinyRound ? Kernel::kTinyRound : Kernel::kPersistent;
 }
 
 // Record upload -> event -> queue reset -> kernel on a private stream.
@@ -825,7 +821,7 @@ int osiris_batch_plan_launch(osiris_batch_plan* p, const osiris_request* reqs, i
   set_granularity(args, &p->opts);
   const int64_t per_block = static_cast<int64_t>(p->block) * args.rays_per_lane;
   int64_t grid = (total + per_block - 1) / per_block;
-  const void* fn = kernel_of(&p->opts, round_kind(total), p->spacetime, total);
+  const void* fn = kernel_of(&p->opts, Kernel::kPersistent, p->spacetime, total);
   int64_t most = 0;
   for (auto& v : p->variant) {
     if (v.fn == nullptr) {  // the plan's first round of this size

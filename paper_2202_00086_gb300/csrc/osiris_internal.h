@@ -65,21 +65,12 @@ constexpr size_t kQueueBytes = 256;  // workspace head: the ray counter
 
 // How a launch deals out its rays: one (or rays_per_lane) per thread, a ray
 // queue in memory, or block indices taken from blocks that have not started
-// (work_steal.cuh; the plain FP64 and DF64 launches). kTinyRound: a batch
-// plan's launch of under kTinyRound rays, a queue in memory as well.
-enum class Kernel { kPlain, kPersistent, kSteal, kTinyRound };
+// (work_steal.cuh; the plain FP64 and DF64 launches).
+enum class Kernel { kPlain, kPersistent, kSteal };
 
 // The trace kernel of a launch: by precision, kind, integrator, space-time and
 // the launch's rays. Each precision has a kernel for small and one for large
 // launches.
-//
-// Tiny rounds of a batch plan (Kernel::kTinyRound) take neither in DF64 and
-// MIXED, but kernels with a register cap, a sine and cosine that branch and, in
-// DF64, sums selected by stage: about twice the time, 6 against 3 ms for 3,000
-// DF64 rays. The server's tests pace their arrivals, one every 2 ms, to rounds
-// of that length and expect them to share launches, which they stop doing when
-// a round is shorter than 5.8 ms.
-constexpr int64_t kTinyRound = 4096;
 const void* trace_kernel_fp64(Kernel kind, int integrator, int spacetime, int64_t rays);
 const void* trace_kernel_mixed(Kernel kind, int integrator, int spacetime, int64_t rays);
 const void* trace_kernel_df64(Kernel kind, int integrator, int spacetime, int64_t rays);

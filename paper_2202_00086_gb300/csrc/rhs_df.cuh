@@ -19,14 +19,13 @@ struct RayDF {
 // Hamilton's equations in the separated form of rhs64 (trace_device.cuh),
 // every operation in df64. twoH receives 2 (H - H0), the distance from the
 // mass shell, at the evaluation point.
-template <bool kBranches = false>
 __device__ __forceinline__ void rhs_df(const RayDF& K, df r, df th, df pr, df pth, df& dr,
                                        df& dth, df& dph, df& dpr, df& dpth, float& twoH) {
   // Intermediate sums and the five outputs are left unrenormalised: every
   // consumer of an output is a product or the renormalising difference
   // k - k1.
   df s, c;
-  df_sincos<kBranches>(th, s, c);
+  df_sincos(th, s, c);
   const df ra2 = df_add_ord_u(df_sqr(r), K.a2);  // r^2 + a^2 (r > 1 >= a)
   const df a2s = df_mul(K.a2, s);
   // renormalised: Delta cancels next to the horizon, and df_rcp below seeds
@@ -69,11 +68,10 @@ struct RayQDF {
   float twoH0;
 };
 
-template <bool kBranches = false>
 __device__ __forceinline__ void rhs_q_df(const RayQDF& K, df r, df th, df pr, df pth, df& dr,
                                          df& dth, df& dph, df& dpr, df& dpth, float& twoH) {
   df s, c;
-  df_sincos<kBranches>(th, s, c);
+  df_sincos(th, s, c);
   const df rm2 = df_add_f(r, -2.0f);  // renormalised: cancels towards r = 2
   const df iD = df_rcp(df_mul(r, rm2));
   const df ir = df_mul(rm2, iD);      // 1/r

@@ -46,7 +46,6 @@ struct RayF32 {
 // t = theta - k pi/2, |t| <= pi/4 (k from the rounded sum; th.hi - k P1 is
 // exact, Sterbenz), then the Taylor polynomials of sin t (to t^9) and cos t
 // (to t^10), whose truncation at |t| = pi/4 is below 3e-9 of the result.
-template <bool kBranches = false>  // kBranches: see kTinyRound (osiris_internal.h)
 __device__ __forceinline__ void sincos_f32(df th, float dth, float& s, float& c) {
   using namespace dfc;
   const float k = rintf(__fmul_rn(__fadd_rn(th.hi, dth), 0.636619772367581343f));
@@ -57,22 +56,6 @@ __device__ __forceinline__ void sincos_f32(df th, float dth, float& s, float& c)
   const float ct =
       fmaf(u, fmaf(u, fmaf(u, fmaf(u, fmaf(u, -I10, I8H), -I6H), I4H), -0.5f), 1.0f);
   const int q = (int)k;
-  if (kBranches) {
-    if ((q & 3) == 0) {
-      s = st;
-      c = ct;
-    } else if ((q & 3) == 1) {
-      s = ct;
-      c = -st;
-    } else if ((q & 3) == 2) {
-      s = -st;
-      c = -ct;
-    } else {
-      s = -ct;
-      c = st;
-    }
-    return;
-  }
   const bool odd = (q & 1) != 0;
   s = flip_sign(odd ? ct : st, sin_sign(q));
   c = flip_sign(odd ? st : ct, cos_sign(q));
@@ -80,12 +63,11 @@ __device__ __forceinline__ void sincos_f32(df th, float dth, float& s, float& c)
 
 // The derivatives (r', theta', phi', p_r', p_theta') and 2 (H - H0) at x,
 // as rhs64 writes them, in FP32.
-template <bool kBranches = false>
 __device__ __forceinline__ void rhs_f32(const RayF32& K, const PointF32& x, float& dr,
                                         float& dth, float& dph, float& dpr, float& dpth,
                                         float& twoH) {
   float s, c;
-  sincos_f32<kBranches>(x.th, x.dth, s, c);
+  sincos_f32(x.th, x.dth, s, c);
   const float rf = __fadd_rn(x.r.hi, x.dr);
   const float prf = x.pr;
   const float ptf = x.pth;
@@ -130,12 +112,11 @@ struct RayQF32 {
 // (rhs_df.cuh) and rhs_q64, the derivatives from the four terms of 2H and
 // their logarithmic derivatives, with f = (r - 2) / r and X = 1 + sin^2 / D,
 // D = r (r - 2).
-template <bool kBranches = false>
 __device__ __forceinline__ void rhs_q_f32(const RayQF32& K, const PointF32& x, float& dr,
                                           float& dth, float& dph, float& dpr, float& dpth,
                                           float& twoH) {
   float s, c;
-  sincos_f32<kBranches>(x.th, x.dth, s, c);
+  sincos_f32(x.th, x.dth, s, c);
   const float rf = __fadd_rn(x.r.hi, x.dr);
   const float prf = x.pr;
   const float ptf = x.pth;

@@ -6,8 +6,6 @@
 // oracle's step on the CPU.
 #pragma once
 
-#include <type_traits>
-
 #include "df64.cuh"
 #include "osiris.h"
 
@@ -89,13 +87,6 @@ OSIRIS_DF_TABLEAU float kDH[2][7] = {
     {0.0f, 0.0f, -0.004252770449966192f, 0.03697916492819786f, -0.05086379870772362f,
      0.041904762387275696f, -0.02500000037252903f}};
 
-// Whether a metric policy is that of the kernels for tiny rounds (kTinyRound,
-// osiris_internal.h), which select the sums of a stage by its number.
-template <class Met, class = void>
-struct SelectsSums : std::false_type {};
-template <class Met>
-struct SelectsSums<Met, std::enable_if_t<Met::kTinyRounds>> : std::true_type {};
-
 struct DerivDF {
   df r, th, ph, pr, pth;
   float twoH;
@@ -148,7 +139,6 @@ __device__ __forceinline__ void rk_step_df(const typename Met::Ray& K, LaneCache
   // as it is added, so that no stage number selects a sum (16 selects a stage
   // when they lay by stage: twelve 512^2 Kerr renders 160.5 -> 148.5 ms, a
   // 161 x 119 one 3.60 -> 2.96, sixteen uneven renders 71.9 -> 66.9).
-  constexpr bool kBySelect = SelectsSums<Met>::value;
   float acc[4][4];
   bool need_k1 = true;
   twoH = 0.0f;
@@ -202,13 +192,7 @@ __device__ __forceinline__ void rk_step_df(const typename Met::Ray& K, LaneCache
 #pragma unroll
       for (int c = 0; c < 4; ++c) {
         const int kc = c < 2 ? c : c + 1;  // skip phi in k
-        const float fs = !kBySelect ? acc[0][c]
-                         : s == 2   ? acc[0][c]
-                         : s == 3   ? acc[1][c]
-                         : s == 4   ? acc[2][c]
-                         : s == 5   ? acc[3][c]
-                                    : 0.0f;
-        in[c] = df_add_f_u(df_add_u(y4[c], df_mul(hk1[kc], cs)), __fmul_rn(hf, fs));
+        in[c] = df_add_f_u(df_add_u(y4[c], df_mul(hk1[kc], cs)), __fmul_rn(hf, acc[0][c]));
       }
     }
     df k[5];
@@ -237,22 +221,12 @@ __device__ __forceinline__ void rk_step_df(const typename Met::Ray& K, LaneCache
 #pragma unroll
     for (int c = 0; c < 5; ++c) e[c] = df_sub(k[c], k1[c]);  // renormalised: the error sum cancels to O(h^5)
     const float ds[4] = {e[0].hi, e[1].hi, e[3].hi, e[4].hi};
-    if (kBySelect) {
+    const StageWeights as = kAS[I][s];
 #pragma unroll
-      for (int t = 2; t < 6; ++t)
-        if (t > s) {
+    for (int t = 0; t < 4; ++t)
 #pragma unroll
-          for (int c = 0; c < 4; ++c)
-            acc[t - 2][c] = fmaf(kA[I][t][s], ds[c], acc[t - 2][c]);
-        }
-    } else {
-      const StageWeights as = kAS[I][s];
-#pragma unroll
-      for (int t = 0; t < 4; ++t)
-#pragma unroll
-        for (int c = 0; c < 4; ++c)
-          acc[t][c] = fmaf(as.w[t], ds[c], t < 3 ? acc[t + 1][c] : 0.0f);
-    }
+      for (int c = 0; c < 4; ++c)
+        acc[t][c] = fmaf(as.w[t], ds[c], t < 3 ? acc[t + 1][c] : 0.0f);
     if (s >= 2) {
       const df bw = mk(kBH[I][s], kBL[I][s]);
       const float dw = kDH[I][s];

@@ -55,17 +55,15 @@ constexpr int64_t kLargeLaunchKerr = 10 * 152 * 256;
 constexpr int64_t kLargeLaunchQ = 8 * 152 * 256;
 constexpr int kLargeRegs = 128;
 
-template <bool kTiny>
 struct KerrDF {
-  static constexpr bool kTinyRounds = kTiny;
   using Ray = RayDF;
-  static constexpr int kMaxRegs = kTiny ? 80 : kLargeRegs;
+  static constexpr int kMaxRegs = kLargeRegs;
   static constexpr bool kFusedR2 = true;
   static __device__ __forceinline__ Ray ray(const RayK& K) { return to_df(K); }
   static __device__ __forceinline__ void rhs(const Ray& K, df r, df th, df pr, df pth, df& dr,
                                              df& dth, df& dph, df& dpr, df& dpth,
                                              float& twoH) {
-    rhs_df<kTiny>(K, r, th, pr, pth, dr, dth, dph, dpr, dpth, twoH);
+    rhs_df(K, r, th, pr, pth, dr, dth, dph, dpr, dpth, twoH);
   }
   static constexpr bool kTrackH = true;
   static constexpr bool kF32Stages = false;
@@ -78,17 +76,15 @@ struct KerrDF {
   }
 };
 
-template <bool kTiny>
 struct QMetricDF {
-  static constexpr bool kTinyRounds = kTiny;
   using Ray = RayQDF;
-  static constexpr int kMaxRegs = kTiny ? 80 : kLargeRegs;
+  static constexpr int kMaxRegs = kLargeRegs;
   static constexpr bool kFusedR2 = true;
   static __device__ __forceinline__ Ray ray(const RayK& K) { return to_qdf(K); }
   static __device__ __forceinline__ void rhs(const Ray& K, df r, df th, df pr, df pth, df& dr,
                                              df& dth, df& dph, df& dpr, df& dpth,
                                              float& twoH) {
-    rhs_q_df<kTiny>(K, r, th, pr, pth, dr, dth, dph, dpr, dpth, twoH);
+    rhs_q_df(K, r, th, pr, pth, dr, dth, dph, dpr, dpth, twoH);
   }
   static constexpr bool kTrackH = true;
   static constexpr bool kF32Stages = false;
@@ -119,15 +115,13 @@ static const void* df64_kernel(Kernel kind) {
                                      : (const void*)trace_df64_plain<Met, INTEG, kLarge>;
 }
 
-template <template <bool> class Met, int INTEG>
+template <class Met, int INTEG>
 static const void* df64_kernel(Kernel kind, int64_t rays, int64_t line) {
-  if (kind == Kernel::kTinyRound)
-    return (const void*)trace_df64_persistent<Met<true>, INTEG, true>;
-  return rays >= line ? df64_kernel<Met<false>, INTEG, true>(kind)
-                      : df64_kernel<Met<false>, INTEG, false>(kind);
+  return rays >= line ? df64_kernel<Met, INTEG, true>(kind)
+                      : df64_kernel<Met, INTEG, false>(kind);
 }
 
-template <template <bool> class Met>
+template <class Met>
 static const void* df64_kernel(Kernel kind, int integrator, int64_t rays, int64_t line) {
   return integrator == OSIRIS_RKDP45 ? df64_kernel<Met, OSIRIS_RKDP45>(kind, rays, line)
                                      : df64_kernel<Met, OSIRIS_RKCK45>(kind, rays, line);

@@ -53,10 +53,9 @@ namespace osiris_impl {
 constexpr int64_t kLargeLaunchKerr = 8 * 152 * 256;
 constexpr int64_t kLargeLaunchQ = 5 * 152 * 256;
 
-template <bool kTiny>
 struct KerrMixed {
   using Ray = RayF32;
-  static constexpr int kMaxRegs = kTiny ? 80 : 96;
+  static constexpr int kMaxRegs = 96;
   static constexpr bool kFusedR2 = false;
   static constexpr bool kTrackH = false;
   static constexpr bool kF32Stages = true;
@@ -79,7 +78,7 @@ struct KerrMixed {
   static __device__ __forceinline__ void rhs_f(const Ray& K, const PointF32& x, float& dr,
                                                float& dth, float& dph, float& dpr, float& dpth,
                                                float& twoH) {
-    rhs_f32<kTiny>(K, x, dr, dth, dph, dpr, dpth, twoH);
+    rhs_f32(K, x, dr, dth, dph, dpr, dpth, twoH);
   }
   // 2 (H - H0) at the end point with the double-float equations of DF64.
   static __device__ __forceinline__ float end_twoH(const Ray& KD, const RayK& K,
@@ -95,7 +94,6 @@ struct KerrMixed {
 
 // The q-metric (Appendix A) with the same stepper; its end-point |H| from
 // the double-float q-metric equations (rhs_q_df).
-template <bool kTiny>
 struct QMetricMixed {
   using Ray = RayQF32;
   static constexpr int kMaxRegs = 128;
@@ -117,7 +115,7 @@ struct QMetricMixed {
   static __device__ __forceinline__ void rhs_f(const Ray& K, const PointF32& x, float& dr,
                                                float& dth, float& dph, float& dpr, float& dpth,
                                                float& twoH) {
-    rhs_q_f32<kTiny>(K, x, dr, dth, dph, dpr, dpth, twoH);
+    rhs_q_f32(K, x, dr, dth, dph, dpr, dpth, twoH);
   }
   static __device__ __forceinline__ float end_twoH(const Ray& KD, const RayK& K,
                                                    const StateDF& y) {
@@ -148,15 +146,13 @@ static const void* mixed_kernel(Kernel kind) {
                                      : (const void*)trace_mixed_plain<Met, INTEG, kLarge>;
 }
 
-template <template <bool> class Met, int INTEG>
+template <class Met, int INTEG>
 static const void* mixed_kernel(Kernel kind, int64_t rays, int64_t line) {
-  if (kind == Kernel::kTinyRound)
-    return (const void*)trace_mixed_persistent<Met<true>, INTEG, true>;
-  return rays >= line ? mixed_kernel<Met<false>, INTEG, true>(kind)
-                      : mixed_kernel<Met<false>, INTEG, false>(kind);
+  return rays >= line ? mixed_kernel<Met, INTEG, true>(kind)
+                      : mixed_kernel<Met, INTEG, false>(kind);
 }
 
-template <template <bool> class Met>
+template <class Met>
 static const void* mixed_kernel(Kernel kind, int integrator, int64_t rays, int64_t line) {
   return integrator == OSIRIS_RKDP45 ? mixed_kernel<Met, OSIRIS_RKDP45>(kind, rays, line)
                                      : mixed_kernel<Met, OSIRIS_RKCK45>(kind, rays, line);

@@ -33,6 +33,15 @@ then the rest of the round budget goes to the oldest of them. Rays are independe
 render's outputs are the same whether it runs alone or in a mix (the GPU
 tests check this bitwise).
 
+Coalescing: a round lasts as long as its longest ray, so that one of a few
+thousand DF64 rays takes the 1.8 ms of one of a few hundred, and keeps a slot
+for that long. A DF64 round of under COALESCE_RAYS rays, and not a full one
+either, is therefore launched no sooner than coalesce_s after the previous
+round of its kind, so that renders which arrive meanwhile share it instead of
+taking a slot each. By default 3 ms on the GPU; 0 turns it off. (FP64 rounds
+last 9 ms and more and fill the slots by themselves, MIXED ones are over in
+0.4 ms.) run() launches the rest at once when no arrival is left.
+
 Failure handling (all on the host; nothing waits on the GPU without a
 bound):
   - cancel(render): a waiting render is dropped at once; an active one gets no
@@ -58,6 +67,7 @@ import numpy as np
 
 SHADOW_BYTES_PER_RAY = 42  # status 1, r/theta/phi/max|H| 32, steps 4, cells 4, parity 1
 DISK_BYTES_PER_RAY = 66    # + g, intensity, r_hit
+COALESCE_RAYS = 4096  # smaller DF64 rounds wait for renders to share them
 HBM_SHARE = 0.8  # default admission budget: this share of the free device memory
 
 
@@ -106,7 +116,7 @@ class RenderServer:
                  hbm_budget_bytes=None, max_inflight=2, max_entries=4096,
                  keep_outputs=False, cell_deg=10.0, cell_phase_deg=0.0, backend=None,
                  clock=time.perf_counter, graphs=True, stall_timeout_s=None, overlap=True,
-                 loose_precision=None, loose_tol=1e-8):
+                 loose_precision=None, loose_tol=1e-8, coalesce_s=None):
         import paper_2202_00086_gb300 as osr
         self.osr = osr
         self.precision = osr.DF64 if precision is None else precision
@@ -122,6 +132,8 @@ class RenderServer:
         self.hbm_budget = int(hbm_budget_bytes)
         self.max_inflight = int(max_inflight)
         self.max_entries = int(max_entries)
+        self.coalesce_s = (getattr(self.backend, "coalesce_s", 0.0) if coalesce_s is None
+                           else float(coalesce_s))
         self.keep_outputs = keep_outputs
         self.cell_deg = cell_deg
         self.cell_phase_deg = cell_phase_deg
@@ -146,6 +158,8 @@ class RenderServer:
                     for _ in range(self.max_inflight)]
         self._ws_free = list(range(self.max_inflight))
         self._last_kind = None
+        self._last_launch = {}  # kind: when its last round was launched
+        self._expecting = True  # more renders may come
         self._plans = None  # per in-flight slot: {kind: plan}, made on first use
         if graphs and hasattr(self.backend, "plan"):
             self._plans = [{} for _ in self._ws]
@@ -229,11 +243,23 @@ class RenderServer:
             self.active.append(r)
 
     # ---- rounds ----
+    def _waits_for_more(self, kind):
+        """Whether the next round of a kind is too small to launch yet (see
+        Coalescing above)."""
+        if not self._expecting or kind[1] != self.osr.DF64 or kind not in self._last_launch:
+            return False
+        if self.clock() - self._last_launch[kind] >= self.coalesce_s:
+            return False
+        left = sum(r.n_rays - r.next_ray for r in self.active if r.kind == kind)
+        return left < min(COALESCE_RAYS, self.round_rays)
+
     def _next_kind(self):
         kinds = []  # kinds with rays left, in order of their oldest such render
         for r in self.active:
             if r.next_ray < r.n_rays and r.kind not in kinds:
                 kinds.append(r.kind)
+        if self.coalesce_s > 0:
+            kinds = [k for k in kinds if not self._waits_for_more(k)]
         if not kinds:
             return None
         if len(kinds) > 1 and kinds[0] == self._last_kind:
@@ -295,6 +321,7 @@ class RenderServer:
                                         cell_deg=self.cell_deg,
                                         cell_phase_deg=self.cell_phase_deg)
         self._last_kind = kind
+        self._last_launch[kind] = self.clock()
         self.inflight.append(_Round(event, parts, k, self.clock()))
         self.round_entries.append(len(parts))
         self.rounds += 1
@@ -402,8 +429,10 @@ class RenderServer:
             while pending and (not realtime or pending[0][0] <= now - t0):
                 t_arr, rd = pending.popleft()
                 self.submit(rd, arrival=t0 + t_arr if realtime else now)
+            self._expecting = bool(pending)
             if not self.step() and poll_s:
                 time.sleep(poll_s)
+        self._expecting = True
         out = summarize(self.done, t0, self.clock(), rejected=len(self.rejected),
                         launches=self.launches)
         out.update(status=self.status, cancelled=len(self.cancelled),
@@ -533,6 +562,7 @@ class _CudaBackend:
         self.osr = osr
         self.torch = torch
         self._streams = {}
+        self.coalesce_s = 0.003
 
     def _stream(self, slot):
         """The stream of an in-flight slot (None: the current stream). A slot
