@@ -672,8 +672,7 @@ struct osiris_batch_plan {
   int32_t max_requests = 0;
   int32_t spacetime = OSIRIS_SPACETIME_KERR;
   int block = 0;
-  // the kernels that this plan has launched (of a small and a large round),
-  // each with its full grid
+  // the kernels of a small and of a large round, each with its full grid
   struct {
     const void* fn;
     int64_t full_grid;
@@ -777,7 +776,16 @@ int osiris_batch_plan_create(osiris_batch_plan** out, int32_t max_requests, int3
   p->dev_table = reinterpret_cast<ReqDev*>(static_cast<char*>(opts->workspace) +
                                            osiris_impl::kQueueBytes);
   p->block = block_of(&p->opts);
+  // Here and not at the first launch of either size: the query loads the
+  // kernel, and a plan may be made ahead of the time that its launches have.
   int rc = OSIRIS_OK;
+  for (int k = 0; k < 2 && rc == OSIRIS_OK; ++k) {
+    p->variant[k].fn = kernel_of(&p->opts, Kernel::kPersistent, spacetime, k ? INT64_MAX : 1);
+    if (k == 1 && p->variant[1].fn == p->variant[0].fn)
+      p->variant[1] = p->variant[0];
+    else
+      rc = full_grid(&p->opts, p->variant[k].fn, &p->variant[k].full_grid);
+  }
   if (rc == OSIRIS_OK &&
       cudaMallocHost(&p->staging, sizeof(ReqDev) * static_cast<size_t>(max_requests)) !=
           cudaSuccess) {
@@ -822,17 +830,7 @@ int osiris_batch_plan_launch(osiris_batch_plan* p, const osiris_request* reqs, i
   const int64_t per_block = static_cast<int64_t>(p->block) * args.rays_per_lane;
   int64_t grid = (total + per_block - 1) / per_block;
   const void* fn = kernel_of(&p->opts, Kernel::kPersistent, p->spacetime, total);
-  int64_t most = 0;
-  for (auto& v : p->variant) {
-    if (v.fn == nullptr) {  // the plan's first round of this size
-      if (int rc = full_grid(&p->opts, fn, &v.full_grid)) return rc;
-      v.fn = fn;
-    }
-    if (v.fn == fn) {
-      most = v.full_grid;
-      break;
-    }
-  }
+  const int64_t most = p->variant[fn == p->variant[0].fn ? 0 : 1].full_grid;
   if (grid > most) grid = most;
   cudaKernelNodeParams k = p->kernel;
   k.func = const_cast<void*>(fn);
