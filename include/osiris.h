@@ -117,10 +117,14 @@ typedef struct {
                               that may run at the same time. */
     size_t workspace_bytes;
     int32_t integrator;    /* OSIRIS_RKCK45 (default) or OSIRIS_RKDP45 */
-    int32_t rays_per_lane; /* rays a lane takes at once, 0..64 (0 = 1): a plain
-                              launch deals out this many consecutive pixels
-                              per thread at a time; a persistent grid claims
-                              this many per idle lane with each queue atomic */
+    int32_t rays_per_lane; /* 0..64 (0 = 1). Persistent grid: rays that each idle
+                              lane claims with a queue atomic. Plain launch in
+                              OSIRIS_MIXED: consecutive pixels of each thread.
+                              Plain launch in OSIRIS_FP64 or OSIRIS_DF64: every
+                              lane takes one ray at a time, and this many times
+                              32 (in small launches times a block's threads)
+                              consecutive pixels make a unit of work that a
+                              block takes over whole */
     int32_t refill_lanes;  /* persistent grid, 0..32 (0 = library default: 4,
                               32 in OSIRIS_MIXED): a
                               warp whose other lanes are still integrating

@@ -222,7 +222,8 @@ int launch(KernelArgs& args, const osiris_trace_opts* o, void* stream) {
     if (needed > 0x7fffffff) return OSIRIS_EINVAL;
     args.queue = nullptr;
     int64_t grid = needed;
-    if (o->precision != OSIRIS_MIXED) {  // plain FP64 and DF64 kernels steal (work_steal.cuh)
+    const Kernel kind = o->precision == OSIRIS_MIXED ? Kernel::kPlain : Kernel::kSteal;
+    if (kind == Kernel::kSteal) {
       const int64_t small_chunk = kStealChunk * args.rays_per_lane;
       args.chunk = args.total_rays > kStealFrom &&
                            args.total_rays <= small_chunk * int64_t{0x7fffffff}
@@ -236,8 +237,7 @@ int launch(KernelArgs& args, const osiris_trace_opts* o, void* stream) {
               cudaSuccess)
         return OSIRIS_ECUDA;
     }
-    return launch_kernel(kernel_of(o, Kernel::kPlain, spacetime, args.total_rays), args, grid,
-                         block, s);
+    return launch_kernel(kernel_of(o, kind, spacetime, args.total_rays), args, grid, block, s);
   }
   if (!o->workspace || o->workspace_bytes < osiris_impl::kQueueBytes) return OSIRIS_ENOMEM;
   const void* fn = kernel_of(o, Kernel::kPersistent, spacetime, args.total_rays);

@@ -54,7 +54,8 @@ struct KernelArgs {
   int64_t total_rays;
   unsigned long long* queue;       // persistent grids: next ray index (device)
   unsigned long long* stats;       // optional OSIRIS_STATS_LEN counters (device)
-  int32_t rays_per_lane;           // rays a lane claims at once (plain: per thread), >= 1
+  int32_t rays_per_lane;           // rays a lane claims at once (plain: per thread; stealing:
+                                   // only in `chunk`), >= 1
   int32_t refill_lanes;            // persistent, stealing: idle lanes a warp waits for before
                                    // it refills (unless none of its lanes is busy), 1..32
   int64_t chunk;                   // stealing: rays that a block index stands for
@@ -63,9 +64,11 @@ struct KernelArgs {
 
 constexpr size_t kQueueBytes = 256;  // workspace head: the ray counter
 
-// How a launch deals out its rays: one (or rays_per_lane) per thread, a ray
-// queue in memory, or block indices taken from blocks that have not started
-// (work_steal.cuh; the plain FP64 and DF64 launches).
+// How a launch deals out its rays: rays_per_lane consecutive ones per thread
+// (kPlain, the plain MIXED launches), a ray queue in memory (kPersistent), or
+// one at a time to each lane that asks, from block indices taken from blocks
+// that have not started (kSteal, work_steal.cuh, the plain FP64 and DF64
+// launches). The kernels of kPlain and kSteal are called trace_*_plain.
 enum class Kernel { kPlain, kPersistent, kSteal };
 
 // The trace kernel of a launch: by precision, kind, integrator, space-time and

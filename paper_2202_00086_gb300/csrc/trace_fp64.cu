@@ -147,8 +147,8 @@ __global__ void __maxnreg__(kLarge ? 128 : 255)
 
 template <int INTEG, class Met, bool kLarge>
 static const void* fp64_kernel(Kernel kind) {
-  return kind == Kernel::kPlain ? (const void*)trace_fp64_plain<INTEG, Met, kLarge>
-                                : (const void*)trace_fp64_persistent<INTEG, Met, kLarge>;
+  return kind == Kernel::kPersistent ? (const void*)trace_fp64_persistent<INTEG, Met, kLarge>
+                                     : (const void*)trace_fp64_plain<INTEG, Met, kLarge>;
 }
 
 template <class Met, bool kLarge>

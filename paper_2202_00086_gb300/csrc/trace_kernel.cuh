@@ -242,9 +242,10 @@ __device__ __forceinline__ LaneClaims& lane_claims() {
   return claims;
 }
 
-// The lane's first claim: a plain launch (one launch thread per ray range)
-// gives each thread rays_per_lane consecutive rays from thread index x
-// rays_per_lane; a persistent grid starts with none and refills.
+// The lane's first claim: a plain MIXED launch (Kernel::kPlain) gives each
+// thread rays_per_lane consecutive rays from thread index x rays_per_lane; a
+// persistent grid starts with none and refills; a stealing launch keeps no
+// claims per lane.
 template <Kernel KIND>
 __device__ __forceinline__ void init_claim(const KernelArgs& A) {
   if (KIND == Kernel::kSteal) return steal_init(A);
