@@ -163,6 +163,27 @@ const void* trace_kernel_fp64(Kernel kind, int integrator, int spacetime, int64_
                               : fp64_kernel<KerrMetric, false>(kind, integrator);
 }
 
+// a b and a + c issued as fused multiply-adds, fma(a, b, -0) and fma(a, 1, c), for
+// the probes below. The -0 and 1 come from constant memory, whose values no
+// compiler pass may assume, so that the instruction stays a fused multiply-add.
+// (The trace kernels take theirs from vector registers, arith64.cuh: an operand
+// in constant memory costs the time of a multiply.)
+static __constant__ double kFmaNegZero = -0.0;
+static __constant__ double kFmaOne = 1.0;
+
+__device__ __forceinline__ double mul_as_fma(double a, double b) {
+  double r;
+  asm("fma.rn.f64 %0, %1, %2, %3;" : "=d"(r) : "d"(a), "d"(b), "d"(kFmaNegZero));
+  return r;
+}
+__device__ __forceinline__ double add_as_fma(double a, double c) {
+  double r;
+  asm("fma.rn.f64 %0, %1, %2, %3;" : "=d"(r) : "d"(a), "d"(kFmaOne), "d"(c));
+  return r;
+}
+__device__ __forceinline__ float mul_as_fma(float a, float b) { return a * b; }
+__device__ __forceinline__ float add_as_fma(float a, float c) { return a + c; }
+
 // Roofline probes: kProbeChains independent chains of one arithmetic
 // operation per thread (OP 0: fused multiply-add a = a b + c, 1: multiply
 // a = a b, 2: add a = a + c, 3: the multiply issued as a fused multiply-add
