@@ -49,23 +49,28 @@ ORACLE_SAMPLE_STRIDE = 128  # CPU baseline: every 128th pixel of each render
 E2E_STEPS = 5  # end-to-end leg: steps timed with host copies (wall clock)
 LOOSE_TOL = 1e-8  # the served stream's looser tolerance, where MIXED is meant to run
 # DRAM bytes (read + write) of one FP64 trace launch over the 1024^2 set: ncu
-# capture (one pass) of the timed launch of the current kernel, 47.60 MB read
-# + 528.18 MB written (profiles/trace_fp64_persistent_kerr12x1024_dram.md);
-# the outputs alone are 528.5 MB (42 B per ray).
-FP64_TRAFFIC_BYTES_PER_LAUNCH = 575.78e6
+# capture (one pass) of the timed launch, 108.73 MB read + 42.97 GB written
+# (profiles/trace_fp64_persistent_kerr12x1024_dram.md). The outputs are 528.5 MB
+# of it (42 B per ray); the rest is the stage values of the attempts, which the
+# kernel keeps in local memory and which the L2 writes back: 21 GB/s.
+FP64_TRAFFIC_BYTES_PER_LAUNCH = 43.08e9
+# FP64-unit thread instructions per attempt of the Kerr kernel: ncu capture of
+# trace_fp64_persistent on the 12 renders at 192x192 (1.4163e9 warp instructions
+# x 28.00 active lanes over 1.5383e8 attempts), profiles/trace_persistent_counters.md.
+FP64_UNIT_INST_PER_ATTEMPT = 258
 # FP32-pipe (FMA heavy + lite) thread instructions, and warp instructions of
 # every pipe, per double-float Cash-Karp attempt on the Kerr set: ncu capture
-# of trace_df64_persistent on the 12 renders at 256x256 (3.3035e10 FMA-pipe
-# warp instructions x 28.97 active lanes, and 3.843e10 warp instructions, over
+# of trace_df64_persistent on the 12 renders at 256x256 (3.3031e10 FMA-pipe
+# warp instructions x 28.95 active lanes, and 3.845e10 warp instructions, over
 # 2.7322e8 attempts), profiles/trace_persistent_counters.md.
-DF64_FP32_INST_PER_ATTEMPT = 3503
+DF64_FP32_INST_PER_ATTEMPT = 3500
 DF64_WARP_INST_PER_ATTEMPT = 140.7
 # The same for the MIXED kernel (FP32 evaluations, FP32 stage sums) at tol
 # 1e-8: ncu capture of trace_mixed_persistent on the 12 renders at 256x256
-# (3.5845e9 FMA-pipe warp instructions x 25.87 active lanes, and 5.3165e9 warp
+# (3.5965e9 FMA-pipe warp instructions x 25.94 active lanes, and 5.1985e9 warp
 # instructions, over 1.4642e8 attempts), profiles/trace_persistent_counters.md.
-MIXED_FP32_INST_PER_ATTEMPT = 633
-MIXED_WARP_INST_PER_ATTEMPT = 36.31
+MIXED_FP32_INST_PER_ATTEMPT = 637
+MIXED_WARP_INST_PER_ATTEMPT = 35.50
 
 
 def fp32_roofline(probe, inst_per_attempt, warp_inst_per_attempt, attempts, seconds):
@@ -921,8 +926,11 @@ def main():
     achieved = flops / max(1, kernel_launches) / (per_launch_ms * 1e-3) / 1e12
     peak = peaks["fp64"] if precision == osr.FP64 else peaks["fp32"]
     # The headline roofline: FP64 operations against the FP64 pipe for the FP64
-    # kernels; for DF64 and MIXED, the FP32 pipe and the issue slots they run
-    # on, from instruction counts measured on the Kerr set (else none).
+    # kernels. That is a rate in algorithmic operations: their products are formed
+    # on the integer pipes, so that it may pass 1; beside it the load of the FP64
+    # unit itself, from its instructions per attempt. For DF64 and MIXED, the FP32
+    # pipe and the issue slots they run on. Both from instruction counts measured
+    # on the Kerr set (else none).
     if precision == osr.FP64:
         roofline_main = {
             "bound": "alu", "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
@@ -933,7 +941,13 @@ def main():
             "peak_source": ("pipe probe measured in this process: FP64 fused "
                             "multiply-add, 16 chains per thread, every SM full"),
             "flops_per_launch": flops / max(1, kernel_launches),
-            "f_rhs": f_rhs, "f_step": F_STEP}
+            "f_rhs": f_rhs, "f_step": F_STEP,
+            "counts": ("algorithmic operations; the products run on the integer pipes, "
+                       "so the FP64 unit's rate is no upper bound"),
+            "fp64_unit_frac": (attempts / max(1, kernel_launches) * FP64_UNIT_INST_PER_ATTEMPT
+                               / (per_launch_ms * 1e-3)
+                               / (32 * probe["fp64_fma"]["warp_inst_per_s"])
+                               if args.workload == "kerr" else None)}
     elif args.workload == "kerr":
         mixed = precision == osr.MIXED
         roofline_main = fp32_roofline(
